@@ -734,7 +734,11 @@ __global__ void __launch_bounds__(LPB) k_ysolve(const YBatch<T> yb, int R, int W
 // ---------------------------------------------------------------------------
 // Krylov helpers
 // ---------------------------------------------------------------------------
-constexpr int kRedThreads = 256;
+// A warp's float64 instruction holds the SM's FP64 pipe for 16 cycles, so what a reduction costs is its adds
+// and how many SMs share them.  With 608 blocks of 256 threads, a shuffle tree per vector and the last block's
+// partial sums added by few warps, the tail of a multi-dot took 10 us per eight vectors and the update's last
+// block (2432 partial sums in one warp) 19 us: 49 and 26 us a launch on vectors of 83 k elements, 16 vectors.
+constexpr int kRedThreads = 512;
 constexpr int kGsMaxVec = 264;  // basis vectors one Gram-Schmidt pass takes (restart length <= 256)
 // gsd layout: [0, kGsMaxVec) first-pass coefficients, [kGsMaxVec, 2 kGsMaxVec) second pass, [3 kGsMaxVec, +4)
 // scalars, [kGsFlag] the tensor-core kernels' wait flag (an int), read back with every Gram-Schmidt result
@@ -754,7 +758,7 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 }
 
 // Called by every thread of every block at the end of a reduction kernel, after each block has
-// written partial[j * nb + b] (j < nv, nb = gridDim.x): the block that arrives last sums the
+// written its partial[j * nb + b] (j < nv, nb = gridDim.x): the block that arrives last sums the
 // partials in a fixed order (lane-strided, then a shuffle tree) into out[j] and resets the
 // counter, so the reduction needs neither a second kernel nor a host round trip.
 __device__ void last_block_reduce(const double* partial, int nv, unsigned* counter, double* out) {
@@ -764,17 +768,63 @@ __device__ void last_block_reduce(const double* partial, int nv, unsigned* count
   __syncthreads();
   if (threadIdx.x == 0) ticket = atomicAdd(counter, 1u);
   __syncthreads();
-  if (ticket != (unsigned)(nb - 1)) return;
+  if (ticket != gridDim.x * gridDim.y - 1u) return;
   __threadfence();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
   for (int j = wid; j < nv; j += nw) {
+    const double* pj = partial + (int64_t)j * nb;
     double s = 0.0;
-    for (int b = lane; b < nb; b += 32) s += __ldcg(&partial[(int64_t)j * nb + b]);
+    int b = lane;
+    for (; b + 96 < nb; b += 128) {  // four loads in flight
+      const double p0 = __ldcg(&pj[b]), p1 = __ldcg(&pj[b + 32]), p2 = __ldcg(&pj[b + 64]), p3 = __ldcg(&pj[b + 96]);
+      s += (p0 + p1) + (p2 + p3);
+    }
+    for (; b < nb; b += 32) s += __ldcg(&pj[b]);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) out[j] = s;
   }
   __syncthreads();
   if (threadIdx.x == 0) *counter = 0u;
+}
+
+// Sums eight values over the warp's lanes, each lane keeping half of its values at every exchange: nine adds
+// instead of the 40 of eight shuffle trees.  Lane 4 u (in the bit order below) returns the sum of v[u].
+__device__ __forceinline__ double warp_sum8(double (&v)[8], int lane) {
+#pragma unroll
+  for (int h = 4; h >= 1; h >>= 1) {
+    const bool up = (lane & (4 * h)) != 0;
+#pragma unroll
+    for (int u = 0; u < h; ++u) {
+      const double send = up ? v[u] : v[u + h];
+      const double keep = up ? v[u + h] : v[u];
+      v[u] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * h);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  return v[0];  // of vector lane >> 2
+}
+
+// |c|^2 of a coefficient vector, by the 32 lanes of one warp (the sum is lane 0's)
+__device__ __forceinline__ double warp_norm2(const double* c, int n, int lane) {
+  double s = 0.0;
+  for (int j = lane; j < n; j += 32) s = fma(c[j], c[j], s);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// The block's sums of eight vectors from its threads' values, added in warp order: thread j < nj writes out[j * ldo].
+__device__ __forceinline__ void block_sum8(double (&v)[8], int nj, double (*sh)[kRedThreads / 32], double* out, int64_t ldo) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const double s = warp_sum8(v, lane);
+  if ((lane & 3) == 0) sh[lane >> 2][wid] = s;
+  __syncthreads();
+  if ((int)threadIdx.x < nj) {
+    double r = 0.0;
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) r += sh[threadIdx.x][q];
+    out[(int64_t)threadIdx.x * ldo] = r;
+  }
+  __syncthreads();
 }
 
 // The float with the sign, the exponent and the 20 leading mantissa bits of a double (truncated;
@@ -821,10 +871,9 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many(const double* __restri
   const int64_t lo = (int64_t)blockIdx.x * chunk;
   const int64_t hi = min(npair, lo + chunk);
   const int nt = nv + (extra ? 1 : 0);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const double2* w2 = reinterpret_cast<const double2*>(w);
   const int64_t bs = blockDim.x;
-  for (int j0 = 0; j0 < nt; j0 += JT) {
+  for (int j0 = (int)blockIdx.y * JT; j0 < nt; j0 += JT * (int)gridDim.y) {
     const int nj = min(JT, nt - j0);
     const double2* vp[JT];
 #pragma unroll
@@ -875,19 +924,11 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many(const double* __restri
           else acc[u] = fma(vv[e], w[e], acc[u]);
         }
     }
+    if (LOWP) {
 #pragma unroll
-    for (int u = 0; u < JT; ++u) {
-      double v = LOWP ? (double)accf[u] : acc[u];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) sh[u][wid] = v;
+      for (int u = 0; u < JT; ++u) acc[u] = (double)accf[u];
     }
-    __syncthreads();
-    if ((int)threadIdx.x < nj) {
-      double r = 0.0;
-      for (int q = 0; q < kRedThreads / 32; ++q) r += sh[threadIdx.x][q];
-      partial[(int64_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = r;
-    }
-    __syncthreads();
+    block_sum8(acc, nj, sh, partial + (int64_t)j0 * gridDim.x + blockIdx.x, gridDim.x);
   }
   last_block_reduce(partial, nt, counter, out);
 }
@@ -904,8 +945,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many_s(const double* __rest
   const int64_t lo = (int64_t)blockIdx.x * chunk;
   const int64_t hi = min(n, lo + chunk);
   const int nt = nv + (extra ? 1 : 0);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int j0 = 0; j0 < nt; j0 += JT) {
+  for (int j0 = (int)blockIdx.y * JT; j0 < nt; j0 += JT * (int)gridDim.y) {
     const int nj = min(JT, nt - j0);
     const double* vp[JT];
 #pragma unroll
@@ -929,19 +969,11 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many_s(const double* __rest
           else acc[u] = fma(vp[u][i], wi, acc[u]);
         }
     }
+    if (LOWP) {
 #pragma unroll
-    for (int u = 0; u < JT; ++u) {
-      double v = LOWP ? (double)accf[u] : acc[u];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) sh[u][wid] = v;
+      for (int u = 0; u < JT; ++u) acc[u] = (double)accf[u];
     }
-    __syncthreads();
-    if ((int)threadIdx.x < nj) {
-      double r = 0.0;
-      for (int q = 0; q < kRedThreads / 32; ++q) r += sh[threadIdx.x][q];
-      partial[(int64_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = r;
-    }
-    __syncthreads();
+    block_sum8(acc, nj, sh, partial + (int64_t)j0 * gridDim.x + blockIdx.x, gridDim.x);
   }
   last_block_reduce(partial, nt, counter, out);
 }
@@ -956,8 +988,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many32(const float* __restr
   const int64_t chunk = (n + gridDim.x - 1) / gridDim.x;
   const int64_t lo = (int64_t)blockIdx.x * chunk;
   const int64_t hi = min(n, lo + chunk);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int j0 = 0; j0 < nv; j0 += JT) {
+  for (int j0 = (int)blockIdx.y * JT; j0 < nv; j0 += JT * (int)gridDim.y) {
     const int nj = min(JT, nv - j0);
     float acc[JT];
 #pragma unroll
@@ -968,19 +999,10 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many32(const float* __restr
       for (int u = 0; u < JT; ++u)
         if (u < nj) acc[u] = fmaf(V[(int64_t)(j0 + u) * ldv + i], wi, acc[u]);
     }
+    double accd[JT];
 #pragma unroll
-    for (int u = 0; u < JT; ++u) {
-      double v = (double)acc[u];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) sh[u][wid] = v;
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < nj) {
-      double r = 0.0;
-      for (int q = 0; q < kRedThreads / 32; ++q) r += sh[threadIdx.x][q];
-      partial[(int64_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = r;
-    }
-    __syncthreads();
+    for (int u = 0; u < JT; ++u) accd[u] = (double)acc[u];
+    block_sum8(accd, nj, sh, partial + (int64_t)j0 * gridDim.x + blockIdx.x, gridDim.x);
   }
   last_block_reduce(partial, nv, counter, out);
 }
@@ -1038,8 +1060,9 @@ __global__ void k_axpby32(float a, const float* __restrict__ x, float b, float* 
 // MODE 2 (single pass with the DGKS test): as MODE 1 when nu^2 >= nrm2_prev / 2 (little cancellation: one
 // float64 projection is enough), out[2] = 0; otherwise as MODE 0 (w <- w', out[0] = ||w'||^2) with
 // out[2] = 1, and the caller re-orthogonalises.  Every block takes the same decision from the same values.
-template <int MODE>
-__global__ void __launch_bounds__(kRedThreads) k_gs_axpy(const double* __restrict__ V, int64_t ldv, int nv,
+// PAIRS: the vectors are read as 16-byte element pairs (every vector on a 16-byte boundary).
+template <int MODE, bool PAIRS>
+__global__ void __launch_bounds__(kRedThreads, 2) k_gs_axpy(const double* __restrict__ V, int64_t ldv, int nv,
                                                         const double* __restrict__ h, const double* __restrict__ G,
                                                         const double* __restrict__ a, double* w, double* vout,
                                                         int64_t n, double* __restrict__ partial, unsigned* counter,
@@ -1060,19 +1083,20 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_axpy(const double* __restric
     cs[j] = cj;
   }
   __syncthreads();
-  if (MODE >= 1 && threadIdx.x == 0) {
-    double c2 = 0.0;
-    for (int j = 0; j < nv; ++j) c2 = fma(cs[j], cs[j], c2);
-    const double nu2 = *nrm2_prev - c2;
-    const double nu = nu2 > 0.0 ? sqrt(nu2) : 0.0;
-    inv_nu = nu > 0.0 ? 1.0 / nu : 0.0;
-    reorth = (MODE == 2 && !(nu2 >= 0.5 * *nrm2_prev)) ? 1 : 0;
-    // closing update on the FP32 pipe only while |h| <= 1e-5 |w'| (its float32 error, ~1e-7 |V h|, then stays
-    // below 1e-12 |w'|); with heavier cancellation the float64 path below
-    corr32 = (MODE == 1 && c2 <= 1e-10 * *nrm2_prev) ? 1 : 0;
-    if (blockIdx.x == 0) {
-      out[1] = nu;
-      if (MODE == 2) out[2] = (double)reorth;
+  if (MODE >= 1 && threadIdx.x < 32) {
+    const double c2 = warp_norm2(cs, nv, threadIdx.x);
+    if (threadIdx.x == 0) {
+      const double nu2 = *nrm2_prev - c2;
+      const double nu = nu2 > 0.0 ? sqrt(nu2) : 0.0;
+      inv_nu = nu > 0.0 ? 1.0 / nu : 0.0;
+      reorth = (MODE == 2 && !(nu2 >= 0.5 * *nrm2_prev)) ? 1 : 0;
+      // closing update on the FP32 pipe only while |h| <= 1e-5 |w'| (its float32 error, ~1e-7 |V h|, then stays
+      // below 1e-12 |w'|); with heavier cancellation the float64 path below
+      corr32 = (MODE == 1 && c2 <= 1e-10 * *nrm2_prev) ? 1 : 0;
+      if (blockIdx.x == 0) {
+        out[1] = nu;
+        if (MODE == 2) out[2] = (double)reorth;
+      }
     }
   }
   __syncthreads();
@@ -1085,21 +1109,40 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_axpy(const double* __restric
     __shared__ float csf[kGsMaxVec];
     for (int j = threadIdx.x; j < nv; j += blockDim.x) csf[j] = (float)cs[j];
     __syncthreads();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-      float c0 = 0.f, c1 = 0.f;
-      int j = 0;
-      for (; j + 7 < nv; j += 8) {
-        double t[8];
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+    int64_t tail = 0;
+    if (PAIRS) {
+      const int64_t npair = n / 2, ldp = ldv / 2;
+      tail = 2 * npair;
+      const double2* V2 = reinterpret_cast<const double2*>(V);
+      for (int64_t p = i0; p < npair; p += st) {
+        float ca = 0.f, cb = 0.f;
+        int j = 0;
+        for (; j + 7 < nv; j += 8) {
+          double2 t[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) t[u] = V[(int64_t)(j + u) * ldv + i];
+          for (int u = 0; u < 8; ++u) t[u] = V2[(int64_t)(j + u) * ldp + p];
 #pragma unroll
-        for (int u = 0; u < 8; u += 2) {
-          c0 = fmaf(csf[j + u], f64_trunc_f32(t[u]), c0);
-          c1 = fmaf(csf[j + u + 1], f64_trunc_f32(t[u + 1]), c1);
+          for (int u = 0; u < 8; ++u) {
+            ca = fmaf(csf[j + u], f64_trunc_f32(t[u].x), ca);
+            cb = fmaf(csf[j + u], f64_trunc_f32(t[u].y), cb);
+          }
         }
+        for (; j < nv; ++j) {
+          const double2 t = V2[(int64_t)j * ldp + p];
+          ca = fmaf(csf[j], f64_trunc_f32(t.x), ca);
+          cb = fmaf(csf[j], f64_trunc_f32(t.y), cb);
+        }
+        const double2 wp = reinterpret_cast<const double2*>(w)[p];
+        const double oa = (wp.x - (double)ca) * inv_nu, ob = (wp.y - (double)cb) * inv_nu;
+        reinterpret_cast<double2*>(vout)[p] = make_double2(oa, ob);
+        acc = fma(ob, ob, fma(oa, oa, acc));
       }
-      for (; j < nv; ++j) c0 = fmaf(csf[j], f64_trunc_f32(V[(int64_t)j * ldv + i]), c0);
-      const double o = (w[i] - (double)(c0 + c1)) * inv_nu;
+    }
+    for (int64_t i = tail + i0; i < n; i += st) {
+      float c0 = 0.f;
+      for (int j = 0; j < nv; ++j) c0 = fmaf(csf[j], f64_trunc_f32(V[(int64_t)j * ldv + i]), c0);
+      const double o = (w[i] - (double)c0) * inv_nu;
       vout[i] = o;
       acc = fma(o, o, acc);
     }
@@ -1108,27 +1151,46 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_axpy(const double* __restric
     last_block_reduce(partial, 1, counter, out);
     return;
   }
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    // one FMA per basis vector on a single chain (no partial sums to add: FP64 issue is the bound);
-    // eight loads issued ahead of their FMAs
+  // one FMA per basis vector and element on a single chain (no partial sums to add: FP64 issue is the bound);
+  // eight 16-byte loads ahead of their FMAs
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+  int64_t tail = 0;
+  if (PAIRS) {
+    const int64_t npair = n / 2, ldp = ldv / 2;
+    tail = 2 * npair;
+    const double2* V2 = reinterpret_cast<const double2*>(V);
+    for (int64_t p = i0; p < npair; p += st) {
+      double2 v = reinterpret_cast<const double2*>(w)[p];
+      int j = 0;
+      for (; j + 7 < nv; j += 8) {
+        double2 t[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) t[u] = V2[(int64_t)(j + u) * ldp + p];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          v.x = fma(-cs[j + u], t[u].x, v.x);
+          v.y = fma(-cs[j + u], t[u].y, v.y);
+        }
+      }
+      for (; j < nv; ++j) {
+        const double2 t = V2[(int64_t)j * ldp + p];
+        v.x = fma(-cs[j], t.x, v.x);
+        v.y = fma(-cs[j], t.y, v.y);
+      }
+      if (!write_w) {
+        v.x *= inv_nu;
+        v.y *= inv_nu;
+      }
+      reinterpret_cast<double2*>(write_w ? w : vout)[p] = v;
+      acc = fma(v.y, v.y, fma(v.x, v.x, acc));
+    }
+  }
+  for (int64_t i = tail + i0; i < n; i += st) {
     double v = w[i];
-    int j = 0;
-    for (; j + 7 < nv; j += 8) {
-      double t[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) t[u] = V[(int64_t)(j + u) * ldv + i];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) v = fma(-cs[j + u], t[u], v);
-    }
-    for (; j < nv; ++j) v = fma(-cs[j], V[(int64_t)j * ldv + i], v);
-    if (write_w) {
-      w[i] = v;
-      acc = fma(v, v, acc);
-    } else {
-      const double o = v * inv_nu;
-      vout[i] = o;
-      acc = fma(o, o, acc);
-    }
+    for (int j = 0; j < nv; ++j) v = fma(-cs[j], V[(int64_t)j * ldv + i], v);
+    if (!write_w) v *= inv_nu;
+    (write_w ? w : vout)[i] = v;
+    acc = fma(v, v, acc);
   }
   acc = block_sum(acc, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = acc;
@@ -1153,10 +1215,9 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many32v(const float* __rest
   const int64_t chunk = (nq + gridDim.x - 1) / gridDim.x;
   const int64_t lo = (int64_t)blockIdx.x * chunk;
   const int64_t hi = min(nq, lo + chunk);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const float4* w4 = reinterpret_cast<const float4*>(w);
   const int64_t bs = blockDim.x;
-  for (int j0 = 0; j0 < nv; j0 += JT) {
+  for (int j0 = (int)blockIdx.y * JT; j0 < nv; j0 += JT * (int)gridDim.y) {
     const int nj = min(JT, nv - j0);
     const float4* vp[JT];
 #pragma unroll
@@ -1184,27 +1245,26 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many32v(const float* __rest
       for (int u = 0; u < JT; ++u)
         if (u < nj) acc[u] = dot4f(vp[u][p], wa, acc[u]);
     }
+    double accd[JT];
 #pragma unroll
-    for (int u = 0; u < JT; ++u) {
-      double v = (double)acc[u];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) sh[u][wid] = v;
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < nj) {
-      double r = 0.0;
-      for (int q = 0; q < kRedThreads / 32; ++q) r += sh[threadIdx.x][q];
-      partial[(int64_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = r;
-    }
-    __syncthreads();
+    for (int u = 0; u < JT; ++u) accd[u] = (double)acc[u];
+    block_sum8(accd, nj, sh, partial + (int64_t)j0 * gridDim.x + blockIdx.x, gridDim.x);
   }
   last_block_reduce(partial, nv, counter, out);
 }
 
 // w' = w - sum_j h_j V_j (float32, h from the device); MODE 0: w <- w', out[0] = ||w'||^2;
 // MODE 1: vout = w' / nu with nu^2 = nrm2_prev - |h|^2, out[0] = ||vout||^2, out[1] = nu.
-template <int MODE>
-__global__ void __launch_bounds__(kRedThreads) k_gs_axpy32(const float* __restrict__ V, int64_t ldv, int nv,
+// QUADS: 16-byte quads (n a multiple of 4, 16-byte aligned vectors), eight in flight per thread.
+__device__ __forceinline__ void sub4(float4& v, float c, const float4& t) {
+  v.x = fmaf(-c, t.x, v.x);
+  v.y = fmaf(-c, t.y, v.y);
+  v.z = fmaf(-c, t.z, v.z);
+  v.w = fmaf(-c, t.w, v.w);
+}
+
+template <int MODE, bool QUADS>
+__global__ void __launch_bounds__(kRedThreads, 2) k_gs_axpy32(const float* __restrict__ V, int64_t ldv, int nv,
                                                           const double* __restrict__ h, float* w, float* vout,
                                                           int64_t n, double* __restrict__ partial, unsigned* counter,
                                                           double* __restrict__ out,
@@ -1214,34 +1274,46 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_axpy32(const float* __restri
   __shared__ float inv_nu;
   for (int j = threadIdx.x; j < nv; j += blockDim.x) cs[j] = (float)h[j];
   __syncthreads();
-  if (MODE == 1 && threadIdx.x == 0) {
-    double c2 = 0.0;
-    for (int j = 0; j < nv; ++j) c2 = fma(h[j], h[j], c2);
-    const double nu2 = *nrm2_prev - c2;
-    const double nu = nu2 > 0.0 ? sqrt(nu2) : 0.0;
-    inv_nu = nu > 0.0 ? (float)(1.0 / nu) : 0.f;
-    if (blockIdx.x == 0) out[1] = nu;
+  if (MODE == 1 && threadIdx.x < 32) {
+    const double c2 = warp_norm2(h, nv, threadIdx.x);
+    if (threadIdx.x == 0) {
+      const double nu2 = *nrm2_prev - c2;
+      const double nu = nu2 > 0.0 ? sqrt(nu2) : 0.0;
+      inv_nu = nu > 0.0 ? (float)(1.0 / nu) : 0.f;
+      if (blockIdx.x == 0) out[1] = nu;
+    }
   }
   __syncthreads();
   double acc = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    float v = w[i];
-    int j = 0;
-    for (; j + 7 < nv; j += 8) {
-      float t[8];
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, st = (int64_t)gridDim.x * blockDim.x;
+  if (QUADS) {
+    const int64_t nq = n / 4, ldq = ldv / 4;
+    const float4* V4 = reinterpret_cast<const float4*>(V);
+    for (int64_t p = i0; p < nq; p += st) {
+      float4 v = reinterpret_cast<const float4*>(w)[p];
+      int j = 0;
+      for (; j + 7 < nv; j += 8) {
+        float4 t[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) t[u] = V[(int64_t)(j + u) * ldv + i];
+        for (int u = 0; u < 8; ++u) t[u] = V4[(int64_t)(j + u) * ldq + p];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v = fmaf(-cs[j + u], t[u], v);
+        for (int u = 0; u < 8; ++u) sub4(v, cs[j + u], t[u]);
+      }
+      for (; j < nv; ++j) sub4(v, cs[j], V4[(int64_t)j * ldq + p]);
+      if (MODE == 1) v = make_float4(v.x * inv_nu, v.y * inv_nu, v.z * inv_nu, v.w * inv_nu);
+      reinterpret_cast<float4*>(MODE == 1 ? vout : w)[p] = v;
+      acc = fma((double)v.x, (double)v.x, acc);
+      acc = fma((double)v.y, (double)v.y, acc);
+      acc = fma((double)v.z, (double)v.z, acc);
+      acc = fma((double)v.w, (double)v.w, acc);
     }
-    for (; j < nv; ++j) v = fmaf(-cs[j], V[(int64_t)j * ldv + i], v);
-    if (MODE == 0) {
-      w[i] = v;
-      acc += (double)v * (double)v;
-    } else {
-      const float o = v * inv_nu;
-      vout[i] = o;
-      acc += (double)o * (double)o;
+  } else {
+    for (int64_t i = i0; i < n; i += st) {
+      float v = w[i];
+      for (int j = 0; j < nv; ++j) v = fmaf(-cs[j], V[(int64_t)j * ldv + i], v);
+      if (MODE == 1) v *= inv_nu;
+      (MODE == 1 ? vout : w)[i] = v;
+      acc = fma((double)v, (double)v, acc);
     }
   }
   acc = block_sum(acc, sh);
@@ -1372,8 +1444,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many_dd(const dd* __restric
                                                             double* __restrict__ out) {
   constexpr int JT = 8;
   __shared__ double sh[JT][kRedThreads / 32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (int j0 = 0; j0 < nv; j0 += JT) {
+  for (int j0 = (int)blockIdx.y * JT; j0 < nv; j0 += JT * (int)gridDim.y) {
     const int nj = min(JT, nv - j0);
     dd acc[JT];
 #pragma unroll
@@ -1384,19 +1455,10 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many_dd(const dd* __restric
       for (int u = 0; u < JT; ++u)
         if (u < nj) acc[u] = fma(V[(int64_t)(j0 + u) * ldv + i], wi, acc[u]);
     }
+    double accd[JT];
 #pragma unroll
-    for (int u = 0; u < JT; ++u) {
-      double v = dd_d(acc[u]);
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) sh[u][wid] = v;
-    }
-    __syncthreads();
-    if ((int)threadIdx.x < nj) {
-      double r = 0.0;
-      for (int q = 0; q < kRedThreads / 32; ++q) r += sh[threadIdx.x][q];
-      partial[(int64_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = r;
-    }
-    __syncthreads();
+    for (int u = 0; u < JT; ++u) accd[u] = dd_d(acc[u]);
+    block_sum8(accd, nj, sh, partial + (int64_t)j0 * gridDim.x + blockIdx.x, gridDim.x);
   }
   last_block_reduce(partial, nv, counter, out);
 }
@@ -1414,13 +1476,14 @@ __global__ void __launch_bounds__(kRedThreads) k_gs_axpy_dd(const dd* __restrict
   __shared__ double sh[32];
   __shared__ dd inv_nu;
   for (int j = threadIdx.x; j < nv; j += blockDim.x) cs[j] = MODE == 2 ? dd(h[j]) : dd(-h[j]);
-  if (MODE == 1 && threadIdx.x == 0) {
-    double c2 = 0.0;
-    for (int j = 0; j < nv; ++j) c2 = fma(h[j], h[j], c2);
-    const double nu2 = *nrm2_prev - c2;
-    const double nu = nu2 > 0.0 ? sqrt(nu2) : 0.0;
-    inv_nu = nu > 0.0 ? dd(1.0 / nu) : dd(0.f, 0.f);
-    if (blockIdx.x == 0) out[1] = nu;
+  if (MODE == 1 && threadIdx.x < 32) {
+    const double c2 = warp_norm2(h, nv, threadIdx.x);
+    if (threadIdx.x == 0) {
+      const double nu2 = *nrm2_prev - c2;
+      const double nu = nu2 > 0.0 ? sqrt(nu2) : 0.0;
+      inv_nu = nu > 0.0 ? dd(1.0 / nu) : dd(0.f, 0.f);
+      if (blockIdx.x == 0) out[1] = nu;
+    }
   }
   __syncthreads();
   dd acc(0.f, 0.f);
@@ -1446,6 +1509,26 @@ inline int grid_for(int64_t n, int threads, int cap = 152 * 16) {
   if (g > cap) g = cap;
   if (g < 1) g = 1;
   return (int)g;
+}
+
+// Launch shapes of the Gram-Schmidt kernels, n = work items (elements, pairs or quads) per vector.
+// Long vectors: one block of 512 threads per SM for the multi-dots (fewest adds; 18 16-byte loads in flight per
+// thread are enough), two per SM for the updates (8 in flight).  Measured at 3.7 M float64 elements and 30
+// vectors: multi-dot 228 us (252 with two blocks per SM, 294 with four), update 212 us (260 with one, 220 with
+// four).  Short vectors: 256 threads, one pass over the items, and the groups of eight vectors side by side in
+// blockIdx.y (83 k elements, 30 vectors: 16 us; 27 with the groups in turn).
+struct RedShape {
+  dim3 grid;
+  int threads;
+};
+inline RedShape dot_shape(int64_t n, int nv) {
+  if (n >= 152 * 512 * 4) return {dim3(152), 512};
+  const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 511) / 512, 152));
+  return {dim3(nb, std::max(1, std::min((nv + 7) / 8, (304 + nb - 1) / nb))), 256};
+}
+inline RedShape upd_shape(int64_t n) {
+  if (n >= 152 * 512 * 2) return {dim3(304), 512};
+  return {dim3((int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 304))), 256};
 }
 
 }  // namespace
@@ -1787,7 +1870,6 @@ int dot_many_x(fm_ctx* c, const double* V, int64_t ldv, int nv, const double* w,
 // h_dev[j] = V[j] . w (j < nv), h_dev[nv] = extra . w when extra is given; stays on the device
 int dot_many_dev(fm_ctx* c, const double* V, int64_t ldv, int nv, const double* w, const double* extra, double* h_dev,
                  bool lowp) {
-  const int nb = c->red_blocks;
   const int nt = nv + (extra ? 1 : 0);
   if (nt > kGsMaxVec) return FM_ERR_ARG;
   // 16-byte element pairs when every vector starts on a 16-byte boundary, scalar loads otherwise (an odd
@@ -1795,11 +1877,12 @@ int dot_many_dev(fm_ctx* c, const double* V, int64_t ldv, int nv, const double* 
   const uintptr_t al = reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(w) |
                        reinterpret_cast<uintptr_t>(extra) | (uintptr_t)(ldv * 8);
   const bool pairs = (al & 15u) == 0;
+  const RedShape sh = dot_shape(pairs ? c->N / 2 : c->N, nt);
   const int tk_ = prof_begin(c, FM_KERNEL_DOT);
-  if (pairs && lowp) k_dot_many<true><<<nb, kRedThreads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, extra, c->gs_cnt, h_dev);
-  else if (pairs) k_dot_many<false><<<nb, kRedThreads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, extra, c->gs_cnt, h_dev);
-  else if (lowp) k_dot_many_s<true><<<nb, kRedThreads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, extra, c->gs_cnt, h_dev);
-  else k_dot_many_s<false><<<nb, kRedThreads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, extra, c->gs_cnt, h_dev);
+  if (pairs && lowp) k_dot_many<true><<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, extra, c->gs_cnt, h_dev);
+  else if (pairs) k_dot_many<false><<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, extra, c->gs_cnt, h_dev);
+  else if (lowp) k_dot_many_s<true><<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, extra, c->gs_cnt, h_dev);
+  else k_dot_many_s<false><<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, extra, c->gs_cnt, h_dev);
   prof_end(c, tk_, 2.0 * nt * (double)c->N, (nt + 1.0) * 8.0 * (double)c->N);
   c->launches++;
   FM_CUDA(cudaGetLastError());
@@ -1819,6 +1902,22 @@ int axpy_many(fm_ctx* c, const double* V, int64_t ldv, int nv, const double* h_h
   return FM_OK;
 }
 
+// One launch of k_gs_axpy on vectors of stride N: 16-byte pairs when N is even and every buffer allows them.
+template <int MODE>
+static void gs_update(fm_ctx* c, const double* V, int nv, const double* h, const double* G, const double* a, double* w,
+                      double* vout, double* out, const double* nrm2_prev) {
+  const uintptr_t al = reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(w) |
+                       reinterpret_cast<uintptr_t>(vout) | (uintptr_t)(c->N * 8);
+  const bool pairs = (al & 15u) == 0;
+  const RedShape sh = upd_shape(pairs ? c->N / 2 : c->N);
+  if (pairs)
+    k_gs_axpy<MODE, true><<<sh.grid, sh.threads, 0, c->stream>>>(V, c->N, nv, h, G, a, w, vout, c->N, c->red, c->gs_cnt,
+                                                                 out, nrm2_prev);
+  else
+    k_gs_axpy<MODE, false><<<sh.grid, sh.threads, 0, c->stream>>>(V, c->N, nv, h, G, a, w, vout, c->N, c->red, c->gs_cnt,
+                                                                  out, nrm2_prev);
+}
+
 // Classical Gram-Schmidt with one re-orthogonalisation (CGS2) of w against the orthonormal
 // V[0..nv), all coefficients kept on the device:
 //   h1 = V^T w;  w' = w - V h1;  h2 = V^T w';  vout = (w' - V h2) / nu,  nu^2 = ||w'||^2 - |h2|^2.
@@ -1831,21 +1930,18 @@ int gs_cgs2(fm_ctx* c, const double* V, int nv, double* w, double* vout, double*
   double* h1 = c->gsd;
   double* h2 = c->gsd + kGsMaxVec;
   double* sc = c->gsd + 3 * kGsMaxVec;  // [0] ||w'||^2, [1] ||vout||^2, [2] nu
-  const int nb2 = 4 * c->red_blocks;
   int rc;
   // first pass: projections to about 1e-6, on the FP32 pipe; the float64 second pass removes what it leaves
   if ((rc = dot_many_dev(c, V, N, nv, w, nullptr, h1, true))) return rc;
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-    k_gs_axpy<0><<<nb2, kRedThreads, 0, c->stream>>>(V, N, nv, h1, nullptr, nullptr, w, nullptr, N, c->red, c->gs_cnt,
-                                                     sc, nullptr);
+    gs_update<0>(c, V, nv, h1, nullptr, nullptr, w, nullptr, sc, nullptr);
     prof_end(c, tk_, (2.0 * nv + 2.0) * (double)N, (nv + 2.0) * 8.0 * (double)N);
   }
   if ((rc = dot_many_dev(c, V, N, nv, w, nullptr, h2))) return rc;
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-    k_gs_axpy<1><<<nb2, kRedThreads, 0, c->stream>>>(V, N, nv, h2, nullptr, nullptr, w, vout, N, c->red, c->gs_cnt,
-                                                     sc + 1, sc);
+    gs_update<1>(c, V, nv, h2, nullptr, nullptr, w, vout, sc + 1, sc);
     prof_end(c, tk_, (2.0 * nv + 2.0) * (double)N, (nv + 2.0) * 8.0 * (double)N);
   }
   c->launches += 2;
@@ -1879,13 +1975,11 @@ int gs_cgs1(fm_ctx* c, const double* V, int nv, double* w, double* vout, double*
   double* h1 = c->gsd;                  // [nv] V^T w, [nv] |w|^2
   double* h2 = c->gsd + kGsMaxVec;
   double* sc = c->gsd + 3 * kGsMaxVec;  // [1] |out|^2, [2] nu, [3] re-orthogonalise
-  const int nb2 = 4 * c->red_blocks;
   int rc;
   if ((rc = dot_many_dev(c, V, N, nv, w, w, h1))) return rc;
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-    k_gs_axpy<2><<<nb2, kRedThreads, 0, c->stream>>>(V, N, nv, h1, nullptr, nullptr, w, vout, N, c->red, c->gs_cnt,
-                                                     sc + 1, h1 + nv);
+    gs_update<2>(c, V, nv, h1, nullptr, nullptr, w, vout, sc + 1, h1 + nv);
     prof_end(c, tk_, (2.0 * nv + 2.0) * (double)N, (nv + 2.0) * 8.0 * (double)N);
   }
   c->launches++;
@@ -1900,8 +1994,7 @@ int gs_cgs1(fm_ctx* c, const double* V, int nv, double* w, double* vout, double*
     if ((rc = dot_many_dev(c, V, N, nv, w, nullptr, h2))) return rc;
     {
       const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-      k_gs_axpy<1><<<nb2, kRedThreads, 0, c->stream>>>(V, N, nv, h2, nullptr, nullptr, w, vout, N, c->red, c->gs_cnt,
-                                                       sc + 1, sc + 1);
+      gs_update<1>(c, V, nv, h2, nullptr, nullptr, w, vout, sc + 1, sc + 1);
       prof_end(c, tk_, (2.0 * nv + 2.0) * (double)N, (nv + 2.0) * 8.0 * (double)N);
     }
     c->launches++;
@@ -1935,27 +2028,29 @@ int gs_cgs2_32(fm_ctx* c, const float* V, int nv, float* w, float* vout, double*
   double* h1 = c->gsd;
   double* h2 = c->gsd + kGsMaxVec;
   double* sc = c->gsd + 3 * kGsMaxVec;
-  const int nb = c->red_blocks, nb2 = 4 * c->red_blocks;
+  const RedShape sd = dot_shape(quads ? N / 4 : N, nv), su = upd_shape(quads ? N / 4 : N);
   {
     const int tk_ = prof_begin(c, FM_KERNEL_DOT);
-    if (quads) k_dot_many32v<<<nb, kRedThreads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h1);
-    else k_dot_many32<<<nb, kRedThreads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h1);
+    if (quads) k_dot_many32v<<<sd.grid, sd.threads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h1);
+    else k_dot_many32<<<sd.grid, sd.threads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h1);
     prof_end(c, tk_, 2.0 * nv * (double)N, (nv + 1.0) * 4.0 * (double)N);
   }
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-    k_gs_axpy32<0><<<nb2, kRedThreads, 0, c->stream>>>(V, N, nv, h1, w, nullptr, N, c->red, c->gs_cnt, sc, nullptr);
+    if (quads) k_gs_axpy32<0, true><<<su.grid, su.threads, 0, c->stream>>>(V, N, nv, h1, w, nullptr, N, c->red, c->gs_cnt, sc, nullptr);
+    else k_gs_axpy32<0, false><<<su.grid, su.threads, 0, c->stream>>>(V, N, nv, h1, w, nullptr, N, c->red, c->gs_cnt, sc, nullptr);
     prof_end(c, tk_, (2.0 * nv + 2.0) * (double)N, (nv + 2.0) * 4.0 * (double)N);
   }
   {
     const int tk_ = prof_begin(c, FM_KERNEL_DOT);
-    if (quads) k_dot_many32v<<<nb, kRedThreads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h2);
-    else k_dot_many32<<<nb, kRedThreads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h2);
+    if (quads) k_dot_many32v<<<sd.grid, sd.threads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h2);
+    else k_dot_many32<<<sd.grid, sd.threads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h2);
     prof_end(c, tk_, 2.0 * nv * (double)N, (nv + 1.0) * 4.0 * (double)N);
   }
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-    k_gs_axpy32<1><<<nb2, kRedThreads, 0, c->stream>>>(V, N, nv, h2, w, vout, N, c->red, c->gs_cnt, sc + 1, sc);
+    if (quads) k_gs_axpy32<1, true><<<su.grid, su.threads, 0, c->stream>>>(V, N, nv, h2, w, vout, N, c->red, c->gs_cnt, sc + 1, sc);
+    else k_gs_axpy32<1, false><<<su.grid, su.threads, 0, c->stream>>>(V, N, nv, h2, w, vout, N, c->red, c->gs_cnt, sc + 1, sc);
     prof_end(c, tk_, (2.0 * nv + 2.0) * (double)N, (nv + 2.0) * 4.0 * (double)N);
   }
   c->launches += 4;
@@ -1988,9 +2083,7 @@ int tuning_correct(fm_ctx* c, const double* U, const double* WmU, const double* 
   int rc;
   if ((rc = dot_many_dev(c, U, c->N, k, z, nullptr, a))) return rc;
   const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-  k_gs_axpy<0><<<4 * c->red_blocks, kRedThreads, 0, c->stream>>>(WmU, c->N, k, nullptr, Gdev, a, z, nullptr, c->N,
-                                                                 c->red, c->gs_cnt, c->gsd + 3 * kGsMaxVec + 4,
-                                                                 nullptr);
+  gs_update<0>(c, WmU, k, nullptr, Gdev, a, z, nullptr, c->gsd + 3 * kGsMaxVec + 4, nullptr);
   prof_end(c, tk_, 2.0 * k * (double)c->N, (k + 2.0) * 8.0 * (double)c->N);
   c->launches++;
   FM_CUDA(cudaGetLastError());
@@ -2106,11 +2199,11 @@ int prof_harvest(fm_ctx* c) {
 }
 
 int dot_many32(fm_ctx* c, const float* V, int64_t ldv, int nv, const float* w, double* h_host) {
-  const int nb = c->red_blocks;
   if (nv > kGsMaxVec) return FM_ERR_ARG;
+  const RedShape sh = dot_shape(c->N, nv);
   {
     const int tk_ = prof_begin(c, FM_KERNEL_DOT);
-    k_dot_many32<<<nb, kRedThreads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, c->gs_cnt, c->gsd);
+    k_dot_many32<<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, c->gs_cnt, c->gsd);
     prof_end(c, tk_, 2.0 * nv * (double)c->N, (nv + 1.0) * 4.0 * (double)c->N);
   }
   c->launches++;
@@ -2126,10 +2219,10 @@ int axpy_many_norm32(fm_ctx* c, const float* V, int64_t ldv, int nv, const doubl
   std::vector<float> hf(h_host, h_host + nv);
   float* hd = reinterpret_cast<float*>(c->red + (int64_t)c->red_blocks * 256 + 512);
   FM_CUDA(cudaMemcpyAsync(hd, hf.data(), nv * sizeof(float), cudaMemcpyHostToDevice, c->stream));
-  const int nb = 4 * c->red_blocks;
+  const RedShape sh = upd_shape(c->N);
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-    k_axpy_many_norm32<<<nb, kRedThreads, 0, c->stream>>>(V, ldv, nv, hd, sign, w, c->N, c->red, c->gs_cnt,
+    k_axpy_many_norm32<<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, hd, sign, w, c->N, c->red, c->gs_cnt,
                                                           c->gsd + 3 * kGsMaxVec);
     prof_end(c, tk_, (2.0 * nv + 2.0) * (double)c->N, (nv + 2.0) * 4.0 * (double)c->N);
   }
@@ -2228,9 +2321,10 @@ int axpby_dd(fm_ctx* c, double a, const dd* x, double b, dd* y) {
 
 int dot_many_dd(fm_ctx* c, const dd* V, int64_t ldv, int nv, const dd* w, double* h_host) {
   if (nv < 1 || nv > kGsMaxVec) return FM_ERR_ARG;
+  const RedShape sh = dot_shape(c->N, nv);
   {
     const int tk_ = prof_begin(c, FM_KERNEL_DOT);
-    k_dot_many_dd<<<c->red_blocks, kRedThreads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, c->gs_cnt, c->gsd);
+    k_dot_many_dd<<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, c->gs_cnt, c->gsd);
     prof_end(c, tk_, 2.0 * nv * (double)c->N, (nv + 1.0) * 8.0 * (double)c->N);
   }
   c->launches++;
@@ -2245,10 +2339,11 @@ int axpy_many_dd(fm_ctx* c, const dd* V, int64_t ldv, int nv, const double* h_ho
   if (nv < 1 || nv > kGsMaxVec) return FM_ERR_ARG;
   double* hd = c->red + (int64_t)c->red_blocks * 256 + 512;
   FM_CUDA(cudaMemcpyAsync(hd, h_host, nv * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+  const RedShape sh = upd_shape(c->N);
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-    k_gs_axpy_dd<2><<<4 * c->red_blocks, kRedThreads, 0, c->stream>>>(V, ldv, nv, hd, w, nullptr, c->N, nullptr,
-                                                                      nullptr, nullptr, nullptr);
+    k_gs_axpy_dd<2><<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, hd, w, nullptr, c->N, nullptr, nullptr, nullptr,
+                                                           nullptr);
     prof_end(c, tk_, 2.0 * nv * (double)c->N, (nv + 2.0) * 8.0 * (double)c->N);
   }
   c->launches++;
@@ -2264,25 +2359,25 @@ int gs_cgs2_dd(fm_ctx* c, const dd* V, int nv, dd* w, dd* vout, double* h, doubl
   double* h1 = c->gsd;
   double* h2 = c->gsd + kGsMaxVec;
   double* sc = c->gsd + 3 * kGsMaxVec;
-  const int nb = c->red_blocks, nb2 = 4 * c->red_blocks;
+  const RedShape sd = dot_shape(N, nv), su = upd_shape(N);
   {
     const int tk_ = prof_begin(c, FM_KERNEL_DOT);
-    k_dot_many_dd<<<nb, kRedThreads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h1);
+    k_dot_many_dd<<<sd.grid, sd.threads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h1);
     prof_end(c, tk_, 2.0 * nv * (double)N, (nv + 1.0) * 8.0 * (double)N);
   }
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-    k_gs_axpy_dd<0><<<nb2, kRedThreads, 0, c->stream>>>(V, N, nv, h1, w, nullptr, N, c->red, c->gs_cnt, sc, nullptr);
+    k_gs_axpy_dd<0><<<su.grid, su.threads, 0, c->stream>>>(V, N, nv, h1, w, nullptr, N, c->red, c->gs_cnt, sc, nullptr);
     prof_end(c, tk_, (2.0 * nv + 2.0) * (double)N, (nv + 2.0) * 8.0 * (double)N);
   }
   {
     const int tk_ = prof_begin(c, FM_KERNEL_DOT);
-    k_dot_many_dd<<<nb, kRedThreads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h2);
+    k_dot_many_dd<<<sd.grid, sd.threads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h2);
     prof_end(c, tk_, 2.0 * nv * (double)N, (nv + 1.0) * 8.0 * (double)N);
   }
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
-    k_gs_axpy_dd<1><<<nb2, kRedThreads, 0, c->stream>>>(V, N, nv, h2, w, vout, N, c->red, c->gs_cnt, sc + 1, sc);
+    k_gs_axpy_dd<1><<<su.grid, su.threads, 0, c->stream>>>(V, N, nv, h2, w, vout, N, c->red, c->gs_cnt, sc + 1, sc);
     prof_end(c, tk_, (2.0 * nv + 2.0) * (double)N, (nv + 2.0) * 8.0 * (double)N);
   }
   c->launches += 4;
