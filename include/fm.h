@@ -20,8 +20,9 @@
  *    identical (Eq. 2-sym-part), {1, 2, 3} otherwise, {1} in the Schrodinger limit.
  *  - All work is ordered on the context's stream (fm_opts.stream, or the legacy
  *    default stream when NULL).  fm_apply / fm_apply_S return without synchronising;
- *    fm_precond_apply synchronises when its tensor-core stages ran (it reads their wait
- *    flag); fm_solve / fm_eigs synchronise before they return.
+ *    fm_precond_apply synchronises when its float32 tensor-core stages ran (it reads their
+ *    wait flag; the float64 form does not synchronise: a wait that expires there leaves NaN in y and is
+ *    reported by the next fm_solve / fm_eigs); fm_solve / fm_eigs synchronise before they return.
  *  - A context is used by one host thread at a time.
  *  - Energies are in the units of the reduced-coordinate equations (Hartree for
  *    electron-mass units); box sizes R_x, R_y are in reduced Jacobi coordinates.
@@ -105,6 +106,8 @@ enum { FM_PREC_FP64 = 0, FM_PREC_FP32 = 1, FM_PREC_MIXED = 2 };
  * (8 significand bits per operand: a looser preconditioner, the same float64 results) for the z stages
  * and, with n_M = 1, the fused x / y chain; the x stages around the banded y solves (n_M > 1) stay
  * TF32; needs n_x, n_y multiples of 8 in [16, 256] and n_z <= 128 (else FM_ERR_ARG).
+ * Float64 preconditioner (FP64 precision): its z and x mode products run on the tensor cores as exact products
+ * of integer digits (at least float64 accuracy) where n_x and n_z are at most 256; with SIMT on the CUDA cores.
  * On the tensor cores the z stages run as tcgen05 GEMMs when n_z <= 128, and for n_M = 1 the x and y
  * stages of one slab (z mode) run in one kernel that keeps the slab on chip. */
 enum { FM_MMA_AUTO = 0, FM_MMA_SIMT = 1, FM_MMA_TF32 = 2, FM_MMA_BF16 = 3 };

@@ -646,7 +646,7 @@ int fm_create(const fm_system* sys, const fm_grid* grids, int n_grids, const fm_
     if ((rc = dev_alloc(c, (void**)&c->ystage32, (size_t)st * 4))) return fail(rc);
   }
   phase("workspace allocation");
-  if ((rc = tc_setup(c))) return fail(rc);
+  if ((rc = tc_setup(c)) || (rc = f64_setup(c))) return fail(rc);
   phase("tensor maps");
   c->m_alloc = m;
   c->ncv_alloc = o.ncv;
@@ -754,7 +754,8 @@ int fm_precond_apply(fm_ctx* c, const double* x, double* y) {
   if (!c->have_shift) return FM_ERR_NO_SHIFT;
   FM_CUDA(cudaSetDevice(c->device));
   int rc = launch_precond(c, x, y);
-  return rc ? rc : tc_check(c);
+  // the float64 stages are not waited for: a wait that expires there leaves NaN, reported by the next solve
+  return rc || !c->tc_active ? rc : tc_check(c);
 }
 
 int fm_solve(fm_ctx* c, double E, const double* rhs, double* x, fm_info* info) {

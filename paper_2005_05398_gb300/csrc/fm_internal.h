@@ -70,6 +70,13 @@ struct TabsDD {
   dd *zp = nullptr, *W = nullptr, *A = nullptr, *B = nullptr, *iy2 = nullptr, *cval = nullptr, *cw = nullptr;
 };
 
+// A mode-product matrix split into digits for the float64 tensor-core stages (fm_tc64.cu)
+struct F64Mat {
+  CUtensorMap tm;                // digits [nl * 7][n][n padded to 8], float16
+  int* exps = nullptr;           // [nl][n] row exponents
+  const double* W = nullptr;     // the matrices
+};
+
 struct Comp {
   int label = 0;                 // particle label alpha
   int r = 4;                     // taps per point of the component's basis (4 cubic, 6 quintic)
@@ -132,6 +139,7 @@ struct Comp {
   uint16_t *Wx16 = nullptr, *Wxb16 = nullptr, *Wy16 = nullptr, *Wyb16 = nullptr;  // BF16 copies
   CUtensorMap tmz[2];            // W-bar_z, W_z for the z-stage kernel
   CUtensorMap tmf[5];            // fused chain: slab t[slab][j][i], W-bar_x, W-bar_y, W_y, W_x
+  F64Mat f64[4];                 // W-bar_z, W_z, W-bar_x, W_x
   bool tcz = false;              // z stages on the tensor cores
   int tcz_np[2] = {128, 128};    // their tile widths (points per tile), forward / inverse
   int x_pair_ls = 0;             // x pencils (values of l) with complex-conjugate pairs, kept in a real basis
@@ -206,6 +214,7 @@ struct fm_ctx {
   double normH = 0.0, normS = 0.0;  // power-iteration lower bounds of |H|_2 and |S|_2 (0 = not yet estimated)
   bool tc_active = false;        // float32 preconditioner x / y stages on the tensor cores
   bool bf16 = false;             // ... with BF16 operands (z stages and the fused chain), else TF32
+  bool f64_tc = false;           // float64 preconditioner z / x stages on the tensor cores (digit splitting)
   int* tc_err = nullptr;         // device flag: a bounded wait of a tensor-core kernel expired
   int64_t launches = 0;
   int64_t device_bytes = 0;
@@ -282,6 +291,11 @@ int precond_tc_front(fm_ctx* c, const TIO* x, std::vector<Comp*>* banded);
 template <typename TIO>
 int precond_tc_back(fm_ctx* c, TIO* y);                                 // x, z inverse
 bool tc_uses_ydiag(const fm_ctx* c, const Comp& cp);                    // the n_M = 1 y diagonalisation runs
+int f64_setup(fm_ctx* c);      // FM_PREC_FP64: split the z and x matrices (fm_tc64.cu)
+int f64_stage(fm_ctx* c, int stage, const double* in, double* out);
+int64_t f64_digit_bytes(int64_t nl, int n);
+bool encode3t(CUtensorMap* m, const void* ptr, CUtensorMapDataType dt, int esize, int d0, int d1, int d2, int box0,
+              int box1);  // swizzled 3D tensor map
 uint16_t f2bf(float v);                                                 // float -> bfloat16 bits (nearest even)
 }  // namespace fmi
 

@@ -1771,6 +1771,11 @@ static int precond_impl(fm_ctx* c, const TIO* x, TIO* y, T* t) {
   T* u = is32 ? (T*)c->u32 : (T*)c->u64;
   std::vector<fmi::Comp*> banded;
   int rc;
+  // float64 on the tensor cores: z forward, x forward here, x inverse, z inverse below, all components per launch
+  const bool f64 = !is32 && c->f64_tc;
+  if constexpr (std::is_same<T, double>::value && std::is_same<TIO, double>::value) {
+    if (f64 && ((rc = f64_stage(c, 0, x, t)) || (rc = f64_stage(c, 2, t, u)))) return rc;
+  }
   if (tc) {  // z, x and y stages on the tensor cores
     if ((rc = fmi::precond_tc_front<TIO>(c, x, &banded))) return rc;
     if ((rc = ysolve_banded<T>(c, banded, u))) return rc;
@@ -1786,20 +1791,22 @@ static int precond_impl(fm_ctx* c, const TIO* x, TIO* y, T* t) {
     const T* Wxb = std::is_same<T, double>::value ? (const T*)cp.Wxb : (const T*)cp.Wxb32;
     const double ncomp = (double)nxy * cp.nz * c->nM;  // unknowns of this component
     const double ts = (double)sizeof(T);
-    dim3 gz((unsigned)((nxy + 127) / 128), c->nM);
-    const size_t smz = ((size_t)cp.nz * cp.nz + (size_t)cp.nz * 128) * sizeof(T);
-    {
-      const int tk_ = prof_begin(c, FM_KERNEL_ZMIX);
-      k_zmix<TIO, T, T><<<gz, 128, smz, c->stream>>>(Wzb, x, t, cp.nz, nxy, cp.off);
-      prof_end(c, tk_, 2.0 * cp.nz * ncomp, ncomp * (8.0 + ts));
+    if (!f64) {
+      dim3 gz((unsigned)((nxy + 127) / 128), c->nM);
+      const size_t smz = ((size_t)cp.nz * cp.nz + (size_t)cp.nz * 128) * sizeof(T);
+      {
+        const int tk_ = prof_begin(c, FM_KERNEL_ZMIX);
+        k_zmix<TIO, T, T><<<gz, 128, smz, c->stream>>>(Wzb, x, t, cp.nz, nxy, cp.off);
+        prof_end(c, tk_, 2.0 * cp.nz * ncomp, ncomp * (8.0 + ts));
+      }
+      dim3 gx((cp.ny + 63) / 64, (cp.nx + 63) / 64, c->nM * cp.nz);
+      {
+        const int tk_ = prof_begin(c, FM_KERNEL_XMIX);
+        k_mix<T, false, true, false><<<gx, 256, 0, c->stream>>>(Wxb, t, u, cp.nx, cp.ny, cp.nz, cp.off, c->M0, nullptr, nullptr);
+        prof_end(c, tk_, 2.0 * cp.nx * ncomp, 2.0 * ncomp * ts);
+      }
+      c->launches += 2;
     }
-    dim3 gx((cp.ny + 63) / 64, (cp.nx + 63) / 64, c->nM * cp.nz);
-    {
-      const int tk_ = prof_begin(c, FM_KERNEL_XMIX);
-      k_mix<T, false, true, false><<<gx, 256, 0, c->stream>>>(Wxb, t, u, cp.nx, cp.ny, cp.nz, cp.off, c->M0, nullptr, nullptr);
-      prof_end(c, tk_, 2.0 * cp.nx * ncomp, 2.0 * ncomp * ts);
-    }
-    c->launches += 2;
     if (ymda) {
       // n_M = 1: per-l diagonalisation of (A_l, S_y): W_y (Lambda_y + lambda_x)^{-1} W-bar_y on transposed slabs
       const T* Wyb = is32 ? (const T*)cp.Wyb32 : (const T*)cp.Wyb64;
@@ -1821,6 +1828,12 @@ static int precond_impl(fm_ctx* c, const TIO* x, TIO* y, T* t) {
     }
   }
   if ((rc = ysolve_banded<T>(c, banded, u))) return rc;
+  if constexpr (std::is_same<T, double>::value && std::is_same<TIO, double>::value) {
+    if (f64) {
+      if ((rc = f64_stage(c, 3, u, t))) return rc;
+      return f64_stage(c, 1, t, y);
+    }
+  }
   for (auto& cp : c->comps) {
     const int64_t nxy = (int64_t)cp.nx * cp.ny;
     const T* Wz = std::is_same<T, double>::value ? (const T*)cp.Wz : (const T*)cp.Wz32;
@@ -1951,7 +1964,7 @@ int gs_cgs2(fm_ctx* c, const double* V, int nv, double* w, double* vout, double*
                           c->stream));
   FM_CUDA(cudaStreamSynchronize(c->stream));
   const double* hh = c->red_host;
-  if (c->tc_active && reinterpret_cast<const int*>(hh + kGsFlag)[0] != 0) return FM_ERR_TIMEOUT;
+  if (c->tc_err && reinterpret_cast<const int*>(hh + kGsFlag)[0] != 0) return FM_ERR_TIMEOUT;
   for (int i = 0; i < nv; ++i) h[i] = hh[i] + hh[kGsMaxVec + i];
   const double vn2 = hh[3 * kGsMaxVec + 1], nu = hh[3 * kGsMaxVec + 2];
   if (!(nu > 0.0) || !(vn2 > 0.0)) {
@@ -1988,7 +2001,7 @@ int gs_cgs1(fm_ctx* c, const double* V, int nv, double* w, double* vout, double*
                           c->stream));
   FM_CUDA(cudaStreamSynchronize(c->stream));
   const double* hh = c->red_host;
-  if (c->tc_active && reinterpret_cast<const int*>(hh + kGsFlag)[0] != 0) return FM_ERR_TIMEOUT;
+  if (c->tc_err && reinterpret_cast<const int*>(hh + kGsFlag)[0] != 0) return FM_ERR_TIMEOUT;
   for (int i = 0; i < nv; ++i) h[i] = hh[i];
   if (hh[3 * kGsMaxVec + 3] != 0.0) {  // cancellation: second float64 pass on w - V h
     if ((rc = dot_many_dev(c, V, N, nv, w, nullptr, h2))) return rc;
@@ -2002,7 +2015,7 @@ int gs_cgs1(fm_ctx* c, const double* V, int nv, double* w, double* vout, double*
     FM_CUDA(cudaMemcpyAsync(c->red_host, c->gsd, kGsRead * sizeof(double), cudaMemcpyDeviceToHost,
                             c->stream));
     FM_CUDA(cudaStreamSynchronize(c->stream));
-    if (c->tc_active && reinterpret_cast<const int*>(hh + kGsFlag)[0] != 0) return FM_ERR_TIMEOUT;
+    if (c->tc_err && reinterpret_cast<const int*>(hh + kGsFlag)[0] != 0) return FM_ERR_TIMEOUT;
     for (int i = 0; i < nv; ++i) h[i] += hh[kGsMaxVec + i];
   }
   const double vn2 = hh[3 * kGsMaxVec + 1], nu = hh[3 * kGsMaxVec + 2];
@@ -2059,7 +2072,7 @@ int gs_cgs2_32(fm_ctx* c, const float* V, int nv, float* w, float* vout, double*
                           c->stream));
   FM_CUDA(cudaStreamSynchronize(c->stream));
   const double* hh = c->red_host;
-  if (c->tc_active && reinterpret_cast<const int*>(hh + kGsFlag)[0] != 0) return FM_ERR_TIMEOUT;
+  if (c->tc_err && reinterpret_cast<const int*>(hh + kGsFlag)[0] != 0) return FM_ERR_TIMEOUT;
   for (int i = 0; i < nv; ++i) h[i] = hh[i] + hh[kGsMaxVec + i];
   const double vn2 = hh[3 * kGsMaxVec + 1], nu = hh[3 * kGsMaxVec + 2];
   if (!(nu > 0.0) || !(vn2 > 0.0)) {
@@ -2385,7 +2398,7 @@ int gs_cgs2_dd(fm_ctx* c, const dd* V, int nv, dd* w, dd* vout, double* h, doubl
   FM_CUDA(cudaMemcpyAsync(c->red_host, c->gsd, kGsRead * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   FM_CUDA(cudaStreamSynchronize(c->stream));
   const double* hh = c->red_host;
-  if (c->tc_active && reinterpret_cast<const int*>(hh + kGsFlag)[0] != 0) return FM_ERR_TIMEOUT;
+  if (c->tc_err && reinterpret_cast<const int*>(hh + kGsFlag)[0] != 0) return FM_ERR_TIMEOUT;
   for (int i = 0; i < nv; ++i) h[i] = hh[i] + hh[kGsMaxVec + i];
   const double vn2 = hh[3 * kGsMaxVec + 1], nu = hh[3 * kGsMaxVec + 2];
   if (!(nu > 0.0) || !(vn2 > 0.0)) {
