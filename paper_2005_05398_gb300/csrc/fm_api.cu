@@ -611,7 +611,7 @@ int fm_create(const fm_system* sys, const fm_grid* grids, int n_grids, const fm_
   const int m = o.restart_m;
   c->red_blocks = 4 * 152;  // reduction blocks: four per SM
   if ((rc = dev_alloc(c, (void**)&c->P, N * 8)) || (rc = dev_alloc(c, (void**)&c->Q, N * 8)) ||
-      (rc = dev_alloc(c, (void**)&c->R, N * 8)) || (rc = dev_alloc(c, (void**)&c->t64, N * 8)) ||
+      (rc = dev_alloc(c, (void**)&c->t64, N * 8)) ||
       (rc = dev_alloc(c, (void**)&c->u64, N * 8)) || (rc = dev_alloc(c, (void**)&c->t32, N * 4)) ||
       (rc = dev_alloc(c, (void**)&c->u32, N * 4)) || (rc = dev_alloc(c, (void**)&c->V, (size_t)(m + 1) * N * 8)) ||
       (rc = dev_alloc(c, (void**)&c->Z, (size_t)std::max(m, o.ncv) * N * 8)) || (rc = dev_alloc(c, (void**)&c->w, N * 8)) ||
@@ -635,8 +635,7 @@ int fm_create(const fm_system* sys, const fm_grid* grids, int n_grids, const fm_
     if ((rc = dev_alloc(c, (void**)&c->V32, (size_t)(m + 1) * N * 4)) || (rc = dev_alloc(c, (void**)&c->Z32, (size_t)m * N * 4)) ||
         (rc = dev_alloc(c, (void**)&c->w32, N * 4)) || (rc = dev_alloc(c, (void**)&c->r32, N * 4)) ||
         (rc = dev_alloc(c, (void**)&c->d32, N * 4)) || (rc = dev_alloc(c, (void**)&c->e32, N * 4)) ||
-        (rc = dev_alloc(c, (void**)&c->P32, N * 4)) || (rc = dev_alloc(c, (void**)&c->Q32, N * 4)) ||
-        (rc = dev_alloc(c, (void**)&c->R32, N * 4)))
+        (rc = dev_alloc(c, (void**)&c->P32, N * 4)) || (rc = dev_alloc(c, (void**)&c->Q32, N * 4)))
       return fail(rc);
     int64_t st = 0;  // coupling sources regrouped by y interval for the float32 gather
     for (auto& cp : c->comps) {

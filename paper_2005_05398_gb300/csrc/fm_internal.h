@@ -60,14 +60,14 @@ struct Source {          // one V^(s) coupling source of a component (Eq. FM-pre
 
 // float32 copies of the operator tables (mixed-precision inner solves)
 struct Tabs32 {
-  float *Sx = nullptr, *D2x = nullptr, *Sy = nullptr, *D2y = nullptr, *Sz = nullptr, *D1z = nullptr, *D2z = nullptr;
-  float *zp = nullptr, *W = nullptr, *A = nullptr, *B = nullptr, *iy2 = nullptr, *cval = nullptr, *cw = nullptr;
+  float *Sx = nullptr, *D2x = nullptr, *Sy = nullptr, *D2y = nullptr, *zt = nullptr, *qx = nullptr;
+  float *W = nullptr, *iy2 = nullptr, *cval = nullptr, *cw = nullptr;
 };
 
 // double-float copies of the operator tables (mixed_scheme 2: double-float inner solves)
 struct TabsDD {
-  dd *Sx = nullptr, *D2x = nullptr, *Sy = nullptr, *D2y = nullptr, *Sz = nullptr, *D1z = nullptr, *D2z = nullptr;
-  dd *zp = nullptr, *W = nullptr, *A = nullptr, *B = nullptr, *iy2 = nullptr, *cval = nullptr, *cw = nullptr;
+  dd *Sx = nullptr, *D2x = nullptr, *Sy = nullptr, *D2y = nullptr, *zt = nullptr, *qx = nullptr;
+  dd *W = nullptr, *iy2 = nullptr, *cval = nullptr, *cw = nullptr;
 };
 
 // A mode-product matrix split into digits for the float64 tensor-core stages (fm_tc64.cu)
@@ -91,8 +91,11 @@ struct Comp {
   // device tables
   AxisDev dx, dy, dz;
   double* W = nullptr;           // [nM][nz][nx][ny] V_a + sum V^(l)_b + q M'(M'+1) + (J(J+1)-2M'^2)/y^2, q = 1/x^2+1/y^2
-  double* A = nullptr;           // [nz][nx][ny] q (1 - z^2)
-  double* B = nullptr;           // [nM][nz][nx][ny] 2 (M'+1) z q
+  // z taps [nz][1 + 3 nM][r]: S_z, then per M' those of 2 (M'+1) z D1 - (1 - z^2) D2, of the M'+1 coupling
+  // lambda-hat^{J,M'} [2 (M'+1) z S - (1 - z^2) D1] and of the M'-1 coupling lambda-hat^{J,-M'} D1
+  double* zt = nullptr;
+  double* qx = nullptr;          // [nx] 1/x^2
+  int* zf = nullptr;             // [nint_z + 1] first z point of each z interval
   double* iy2 = nullptr;         // [ny] 1/y^2
   // coupling tables: n_act active points, per (source s): taps and weights
   int n_act = 0;
@@ -164,10 +167,9 @@ struct fm_ctx {
   bool have_shift = false;
   double Estar = 0.0;
   // workspace
-  double* P = nullptr;           // [N] y/x-pass planes for the apply (S_x S_y c)
-  double* Q = nullptr;           // [N] (D_x S_y c)
-  double* R = nullptr;           // [N] (S_x D_y c)
-  float* P32 = nullptr; float* Q32 = nullptr; float* R32 = nullptr;  // float32 apply scratch
+  double* P = nullptr;           // [N] planes of the two-pass apply (S_x S_y c)
+  double* Q = nullptr;           // [N] ((D2_x S_y + S_x D2_y) c)
+  float* P32 = nullptr; float* Q32 = nullptr;  // float32 apply scratch
   double* t64 = nullptr;         // [N] preconditioner stage buffer
   double* u64 = nullptr;
   float* t32 = nullptr;
@@ -273,7 +275,7 @@ int fill_normal(fm_ctx* c, double* x, uint64_t seed);
 int combine(fm_ctx* c, const double* V, int64_t ldv, int nv, const double* Q_host, int nc, double* out, int64_t ldo);
 int absmax(fm_ctx* c, const double* x, double* val);
 int kernels_init(fm_ctx* c);
-int launch_apply_scratch(fm_ctx* c, double E, const double* x, double* y, double* P, double* Q, double* R);
+int launch_apply_scratch(fm_ctx* c, double E, const double* x, double* y, double* P, double* Q);
 // timing helpers: begin() returns a token for end(); no-ops unless profiling
 int prof_begin(fm_ctx* c, int cls);
 void prof_end(fm_ctx* c, int token, double flops, double bytes);

@@ -1,8 +1,8 @@
 // CUDA kernels of libfm (sm_103a).
 //
 //  * operator apply y = (H - E S) x (Eq. FM-lin; H from Eq. FM-pre, storage idea of
-//    Eq. l-form): sum-factorised banded contractions, y/x pass then z pass with the
-//    pointwise coefficients and the M' +- 1 couplings fused;
+//    Eq. l-form): sum-factorised banded contractions in y, x and z with the pointwise
+//    coefficients and the M' +- 1 couplings, one kernel that walks the z planes;
 //  * the V^(s) coupling term (Eqs. r-form, s-rot): a gather of the source
 //    component's spline coefficients at the rotated collocation points;
 //  * the tensor-trick preconditioner (Eq. prec-2): z and x mode products and the
@@ -24,159 +24,337 @@ namespace {
 constexpr int kMaxM = 12;  // largest n_M (J <= 11 for tau = +1)
 
 // ---------------------------------------------------------------------------
-// apply, pass 1: for one (component, M', z-dof k) plane c[i][j] (n_x x n_y) and a tile
-// of TX x-collocation points: P = (S_x (x) S_y) c, Q = (D2_x (x) S_y) c, R = (S_x (x) D2_y) c.
-// R taps per point (4 cubic, 6 quintic); the tile reads 'rows' rows of c from the base of its
-// first point (the host sizes 'rows' from the axis' tap structure).
+// The local part of the operator, y = (L - E S) c (or S c).  At a collocation point (zeta, xi, eta) of component M'
+//   y = (W - E) U + q Z - D + (n_M > 1) iy2 [T+ psi_{M'+1} + T- psi_{M'-1}],   q = 1/x^2 + 1/y^2,
+//   U = S_z P,  Z = [2 (M'+1) z D1_z - (1 - z^2) D2_z] P,  D = S_z Q,
+//   P = S_x S_y c,  Q = (D2_x S_y + S_x D2_y) c,
+// with the z contractions' taps combined on the host (cp.zt), so that a point takes 8 (y, times the halo) + 12 (x)
+// + 12 (z) + 3 multiply-adds for r = 4 and n_M = 1 (five separate z contractions and three planes took 45).
+//
+// float32, one pass over the coefficients: a CTA owns a tile of 16 x 16 (x, y) points and a chunk of z intervals
+// and walks the z planes; an interval's planes (with their halo, all M') stream into shared memory by cp.async while
+// the previous ones are contracted in y (shared memory) and x (registers), and every thread keeps the last r planes
+// of P and Q of its point in registers, from which it forms the z outputs of each interval.  The planes never go to
+// memory: 47 us an application at 3.7 M unknowns against 95 us of two kernels (He L = 0, 96 x 96 x 24).
 // ---------------------------------------------------------------------------
-template <int TX, int R, typename T>
-__global__ void __launch_bounds__(256) k_apply_xy(const T* __restrict__ c, T* __restrict__ P,
-                                                  T* __restrict__ Q, T* __restrict__ Rr, int nx, int ny, int rows,
-                                                  const int* __restrict__ bx, const T* __restrict__ Sx,
-                                                  const T* __restrict__ D2x, const int* __restrict__ by,
-                                                  const T* __restrict__ Sy, const T* __restrict__ D2y,
-                                                  bool only_S) {
-  extern __shared__ unsigned char smraw_xy[];
-  T* sm = reinterpret_cast<T*>(smraw_xy);
-  T* cs = sm;                 // [rows][ny]
-  T* As = sm + rows * ny;     // [rows][ny]  S_y pass
-  T* Bs = As + rows * ny;     // [rows][ny]  D2_y pass
-  const int64_t plane = (int64_t)blockIdx.y * nx * ny;
-  const int xi0 = blockIdx.x * TX;
-  const int r0 = bx[xi0];
-  for (int idx = threadIdx.x; idx < rows * ny; idx += blockDim.x) {
-    const int r = r0 + idx / ny;
-    cs[idx] = (r >= 0 && r < nx) ? c[plane + (int64_t)r * ny + (idx % ny)] : (T)0;
+constexpr int kLX = 16, kLY = 16, kLThreads = kLX * kLY;  // tile (points)
+
+struct LocalComp {
+  const float* x;
+  float* y;
+  const float *W, *Sx, *D2x, *Sy, *D2y, *zt, *qx, *iy2;
+  const int *bx, *by, *zf;   // tap bases; first z point of each z interval [nint + 1]
+  int nx, ny, nz;
+  int rows, cols;            // coefficients a tile reads in x and y
+  int tiles_x, tiles_y, nint, q, ipc;  // tiles; z intervals, functions per node, intervals per chunk
+  int first;                 // first block of the component
+};
+struct LocalArgs {
+  LocalComp c[3];
+  int ncomp;
+  float E;
+  int only_S;
+};
+
+template <int B>
+__device__ __forceinline__ void cp_async_elem(void* dst, const void* src, bool ok) {  // zero-filled when !ok
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(d), "l"(src), "n"(B), "r"(ok ? B : 0) : "memory");
+}
+
+template <int R, int NM>
+__global__ void __launch_bounds__(kLThreads, R * NM <= 8 ? 4 : (R * NM <= 12 ? 3 : 2))
+    k_apply_local(const __grid_constant__ LocalArgs a) {
+  using T = float;
+  constexpr int PS = R / 2, kAhead = 2;  // planes per step (an interval); z points whose W is loaded ahead
+  extern __shared__ __align__(16) unsigned char smraw_l[];
+  int ci = 0;
+  while (ci + 1 < a.ncomp && (int)blockIdx.x >= a.c[ci + 1].first) ++ci;
+  const LocalComp& c = a.c[ci];
+  const int rows = c.rows, ld = c.cols + 1, tiles = c.tiles_x * c.tiles_y;
+  T* tab = reinterpret_cast<T*>(smraw_l);       // S_y, D2_y [R][kLY]; S_x, D2_x [R][kLX]
+  T* cs = tab + 2 * R * (kLX + kLY);            // [2][PS][NM][rows][ld]
+  T* As = cs + 2 * PS * NM * rows * ld;         // [PS][NM][rows][kLY]  S_y c
+  T* Bs = As + PS * NM * rows * kLY;            //                      D2_y c
+  const int b = (int)blockIdx.x - c.first, chunk = b / tiles, tile = b - chunk * tiles;
+  const int xi0 = (tile / c.tiles_y) * kLX, eta0 = (tile % c.tiles_y) * kLY;
+  const int tid = threadIdx.x, tx = tid / kLY, ty = tid % kLY;
+  const int xi = xi0 + tx, eta = eta0 + ty;
+  const bool live = xi < c.nx && eta < c.ny;
+  const int xc = min(xi, c.nx - 1), ec = min(eta, c.ny - 1);
+  const int r0 = c.bx[xi0], c0 = c.by[eta0];
+  const int lr = c.bx[xc] - r0, lc = c.by[ec] - c0;
+  for (int e = tid; e < R * (kLX + kLY); e += kLThreads) {
+    const bool isx = e >= R * kLY;
+    const int q = isx ? e - R * kLY : e, n = isx ? kLX : kLY, t = q / n, g = q - t * n;
+    const int at = isx ? min(xi0 + g, c.nx - 1) : min(eta0 + g, c.ny - 1);
+    T* d = tab + (isx ? 2 * R * kLY : 0) + q;
+    d[0] = (isx ? c.Sx : c.Sy)[at * R + t];
+    d[R * n] = (isx ? c.D2x : c.D2y)[at * R + t];
   }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < rows * ny; idx += blockDim.x) {
-    const int r = idx / ny, eta = idx % ny;
-    const int b = by[eta];
-    T a = 0, d = 0;
-#pragma unroll
-    for (int t = 0; t < R; ++t) {
-      const int j = b + t;
-      if (j >= 0 && j < ny) {
-        const T v = cs[r * ny + j];
-        a = fma(Sy[eta * R + t], v, a);
-        d = fma(D2y[eta * R + t], v, d);
+  const T* ys = tab + ty;
+  const T* xs = tab + 2 * R * kLY + tx;
+  const T iy2 = c.iy2[ec], q = c.qx[xc] + iy2;
+  const int64_t nxy = (int64_t)c.nx * c.ny, npts = nxy * c.nz;
+  const int m0 = chunk * c.ipc, m1 = min(c.nint, m0 + c.ipc);
+  const int k0 = c.q * m0, k1 = c.q * (m1 - 1) + R - 1;  // planes of the chunk (their number is a multiple of PS)
+  // rows of PS planes' tiles (all M'), 32 lanes a row
+  auto fetch = [&](int k, int buf) {
+    T* dst = cs + buf * PS * NM * rows * ld;
+    constexpr int LN = 2 * kLY;
+    const int ln = tid % LN;
+    if (ln < c.cols) {
+      const int col = c0 + ln;
+      for (int rr = tid / LN; rr < PS * NM * rows; rr += kLThreads / LN) {
+        const int pm = PS * NM == 1 ? 0 : rr / rows, ps = pm / NM, M = pm - ps * NM, r = r0 + rr - pm * rows;
+        const bool ok = r >= 0 && r < c.nx && col >= 0 && col < c.ny;
+        const T* src = ok ? c.x + ((int64_t)M * c.nz + k + ps) * nxy + (int64_t)r * c.ny + col : c.x;
+        cp_async_elem<sizeof(T)>(dst + rr * ld + ln, src, ok);
       }
     }
-    As[idx] = a;
-    Bs[idx] = d;
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < TX * ny; idx += blockDim.x) {
-    const int xi = xi0 + idx / ny, eta = idx % ny;
-    if (xi >= nx) continue;
-    const int b = bx[xi] - r0;
-    T p = 0, q = 0, rr = 0;
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  T P[NM][R], Q[NM][R];
 #pragma unroll
-    for (int t = 0; t < R; ++t) {
-      const int lr = b + t;
-      if (lr >= 0 && lr < rows) {
-        const T a = As[lr * ny + eta];
-        p = fma(Sx[xi * R + t], a, p);
-        q = fma(D2x[xi * R + t], a, q);
-        rr = fma(Sx[xi * R + t], Bs[lr * ny + eta], rr);
+  for (int M = 0; M < NM; ++M)
+#pragma unroll
+    for (int t = 0; t < R; ++t) P[M][t] = Q[M][t] = (T)0;
+  int m = m0;
+  fetch(k0, 0);
+  const int64_t oxy = (int64_t)xc * c.ny + ec;
+  T wq[kAhead + 1][NM];  // W of the next z points
+  if (!a.only_S) {
+#pragma unroll
+    for (int h = 0; h < kAhead; ++h)
+#pragma unroll
+      for (int M = 0; M < NM; ++M) wq[h][M] = c.W[M * npts + min(c.zf[m0] + h, c.nz - 1) * nxy + oxy];
+  }
+  for (int k = k0, buf = 0; k <= k1; k += PS, buf ^= 1) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // these planes are in shared memory; the previous ones' x pass is done
+    if (k + PS <= k1) fetch(k + PS, buf ^ 1);
+    const T* cb = cs + buf * PS * NM * rows * ld;
+    for (int rr = tx; rr < PS * NM * rows; rr += kLX) {
+      const T* v = cb + rr * ld + lc;
+      T s = ys[0] * v[0], d = ys[R * kLY] * v[0];
+#pragma unroll
+      for (int t = 1; t < R; ++t) {
+        s = fma(ys[t * kLY], v[t], s);
+        d = fma(ys[(R + t) * kLY], v[t], d);
+      }
+      As[rr * kLY + ty] = s;
+      Bs[rr * kLY + ty] = d;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int M = 0; M < NM; ++M) {
+#pragma unroll
+      for (int t = 0; t + PS < R; ++t) {
+        P[M][t] = P[M][t + PS];
+        Q[M][t] = Q[M][t + PS];
+      }
+#pragma unroll
+      for (int ps = 0; ps < PS; ++ps) {
+        const T* pa = As + ((ps * NM + M) * rows + lr) * kLY + ty;
+        const T* pb = Bs + ((ps * NM + M) * rows + lr) * kLY + ty;
+        T p = (T)0, d = (T)0;
+#pragma unroll
+        for (int t = 0; t < R; ++t) {
+          const T av = pa[t * kLY], sx = xs[t * kLX];
+          p = fma(sx, av, p);
+          d = fma(xs[(R + t) * kLX], av, fma(sx, pb[t * kLY], d));
+        }
+        P[M][R - PS + ps] = p;
+        Q[M][R - PS + ps] = d;
       }
     }
-    const int64_t o = plane + (int64_t)xi * ny + eta;
-    P[o] = p;
-    if (!only_S) {
-      Q[o] = q;
-      Rr[o] = rr;
+    if (k + PS - R != c.q * m) continue;
+    // planes q m .. q m + r - 1 are at hand: the z points of interval m
+    const int z1 = c.zf[m + 1];
+    for (int zeta = c.zf[m]; zeta < z1; ++zeta) {
+      const int64_t o = (int64_t)zeta * nxy + oxy;
+      T w[NM];
+      if (!a.only_S) {
+        const int64_t on = min(zeta + kAhead, c.nz - 1) * nxy + oxy;
+#pragma unroll
+        for (int M = 0; M < NM; ++M) {
+          wq[kAhead][M] = c.W[M * npts + on];
+          w[M] = wq[0][M];
+#pragma unroll
+          for (int h = 0; h < kAhead; ++h) wq[h][M] = wq[h + 1][M];
+        }
+      }
+      const T* zt = c.zt + (int64_t)zeta * (1 + 3 * NM) * R;  // S_z, then per M': Z, T+, T- taps
+      T out[NM];
+#pragma unroll
+      for (int M = 0; M < NM; ++M) {
+        T U = zt[0] * P[M][0];
+#pragma unroll
+        for (int t = 1; t < R; ++t) U = fma(zt[t], P[M][t], U);
+        if (a.only_S) {
+          out[M] = U;
+          continue;
+        }
+        const T* zm = zt + (1 + 3 * M) * R;
+        T L = (T)0, D = (T)0;
+#pragma unroll
+        for (int t = 0; t < R; ++t) {
+          L = fma(zm[t], P[M][t], L);
+          D = fma(zt[t], Q[M][t], D);
+        }
+        T v = fma(w[M] - a.E, U, fma(q, L, -D));
+        if (NM > 1) {
+          T e = (T)0;
+          if (M + 1 < NM) {
+#pragma unroll
+            for (int t = 0; t < R; ++t) e = fma(zm[R + t], P[M + 1 < NM ? M + 1 : M][t], e);
+          }
+          if (M > 0) {
+#pragma unroll
+            for (int t = 0; t < R; ++t) e = fma(zm[2 * R + t], P[M > 0 ? M - 1 : M][t], e);
+          }
+          v = fma(iy2, e, v);
+        }
+        out[M] = v;
+      }
+      if (live) {
+#pragma unroll
+        for (int M = 0; M < NM; ++M) c.y[M * npts + o] = out[M];
+      }
+    }
+    ++m;
+  }
+}
+
+// The two-pass form: float64 (bound by its pipe, so what counts is an even spread of the work: k_apply_local's
+// tiles and z chunks cost 5 .. 25 % of it on grids that do not fill them) and n_M beyond the instantiations of
+// k_apply_local.
+// Pass 1: for one (component, M', z-dof k) plane c[i][j] and a tile of 16 x 32 points, the planes
+// P = (S_x (x) S_y) c and Q = (D2_x (x) S_y + S_x (x) D2_y) c.
+constexpr int kPX = 16, kPY = 32;
+template <typename T>
+struct PlaneComp {
+  const T* x;
+  T *P, *Q, *y;
+  const T *W, *Sx, *D2x, *Sy, *D2y, *zt, *qx, *iy2;
+  const int *bx, *by, *bz;
+  int nx, ny, nz, rows, cols, tiles_x, tiles_y;
+  int first_xy, first_z;     // first blocks of the component in the two passes
+};
+template <typename T>
+struct PlaneArgs {
+  PlaneComp<T> c[3];
+  int ncomp, nM;
+  T E;
+  int only_S;
+};
+
+template <int R, typename T>
+__global__ void __launch_bounds__(256) k_apply_xy(const __grid_constant__ PlaneArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char smraw_xy[];
+  int ci = 0;
+  while (ci + 1 < a.ncomp && (int)blockIdx.x >= a.c[ci + 1].first_xy) ++ci;
+  const PlaneComp<T>& c = a.c[ci];
+  const int rows = c.rows, ld = c.cols + 1;
+  T* cs = reinterpret_cast<T*>(smraw_xy);  // [rows][ld]
+  T* As = cs + rows * ld;                  // [rows][kPY]  S_y c
+  T* Bs = As + rows * kPY;                 //              D2_y c
+  const int tiles = c.tiles_x * c.tiles_y, b = (int)blockIdx.x - c.first_xy, pl = b / tiles, tile = b - pl * tiles;
+  const int64_t plane = (int64_t)pl * c.nx * c.ny;
+  const int xi0 = (tile / c.tiles_y) * kPX, eta0 = (tile % c.tiles_y) * kPY;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int eta = eta0 + lane, ec = min(eta, c.ny - 1);
+  const int r0 = c.bx[xi0], c0 = c.by[eta0], lc = c.by[ec] - c0;
+  for (int rr = warp; rr < rows; rr += 8) {
+    const int r = r0 + rr;
+    for (int cc = lane; cc < c.cols; cc += 32) {
+      const int col = c0 + cc;
+      cs[rr * ld + cc] = (r >= 0 && r < c.nx && col >= 0 && col < c.ny) ? c.x[plane + (int64_t)r * c.ny + col] : (T)0;
+    }
+  }
+  T sy[R], dy[R];
+#pragma unroll
+  for (int t = 0; t < R; ++t) {
+    sy[t] = c.Sy[ec * R + t];
+    dy[t] = c.D2y[ec * R + t];
+  }
+  __syncthreads();
+  const int last = min(rows, c.bx[min(xi0 + kPX, c.nx) - 1] + R - r0);  // rows the tile's points read
+  for (int rr = warp; rr < last; rr += 8) {
+    const T* v = cs + rr * ld + lc;
+    T s = sy[0] * v[0], d = dy[0] * v[0];
+#pragma unroll
+    for (int t = 1; t < R; ++t) {
+      s = fma(sy[t], v[t], s);
+      d = fma(dy[t], v[t], d);
+    }
+    As[rr * kPY + lane] = s;
+    Bs[rr * kPY + lane] = d;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int h = 0; h < kPX / 8; ++h) {
+    const int xi = xi0 + warp + 8 * h;
+    if (xi >= c.nx) break;
+    const int lr = c.bx[xi] - r0;
+    T p = 0, q = 0;
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+      const T av = As[(lr + t) * kPY + lane], sx = c.Sx[xi * R + t];
+      p = fma(sx, av, p);
+      q = fma(c.D2x[xi * R + t], av, fma(sx, Bs[(lr + t) * kPY + lane], q));
+    }
+    if (eta < c.ny) {
+      const int64_t o = plane + (int64_t)xi * c.ny + eta;
+      c.P[o] = p;
+      if (!a.only_S) c.Q[o] = q;
     }
   }
 }
 
-template <typename T>
-struct ZPassArgs {
-  const T* P;
-  const T* Q;
-  const T* R;
-  T* y;
-  const T* W;       // [nM][nz][nx][ny] folded diagonal coefficient (without -E)
-  const T* A;       // [nz][nx][ny] (1/x^2 + 1/y^2)(1 - z^2)
-  const T* B;       // [nM][nz][nx][ny] 2 (M'+1) z (1/x^2 + 1/y^2)
-  const T* iy2;     // [ny] 1/y^2
-  const int* bz;
-  const T* Sz;
-  const T* D1z;
-  const T* D2z;
-  const T* zp;
-  int nx, ny, nz, nM, M0, J;
-  T E;
-  T lamp[kMaxM];    // lambda-hat^{J, M'} for M'+1 coupling
-  T lamm[kMaxM];    // lambda-hat^{J, -M'} for M'-1 coupling
-};
-
-// apply, pass 2: one thread per output point (M', zeta, xi, eta) of a component (R taps in z).
+// Pass 2: one thread per output point (M', zeta, xi, eta) (R taps in z).
 template <int R, typename T>
-__global__ void __launch_bounds__(256) k_apply_z(ZPassArgs<T> a, bool only_S) {
-  const int64_t npts = (int64_t)a.nz * a.nx * a.ny;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= npts * a.nM) return;
-  const int iM = (int)(gid / npts);
-  const int64_t pt = gid - (int64_t)iM * npts;
-  const int zeta = (int)(pt / ((int64_t)a.nx * a.ny));
-  const int64_t xy = pt - (int64_t)zeta * a.nx * a.ny;
-  const int b = a.bz[zeta];
-  const int64_t blk = (int64_t)iM * npts;
-  T U = 0, Uz = 0, Uzz = 0, Uxx = 0, Uyy = 0;
+__global__ void __launch_bounds__(256) k_apply_z(const __grid_constant__ PlaneArgs<T> a) {
+  int ci = 0;
+  while (ci + 1 < a.ncomp && (int)blockIdx.x >= a.c[ci + 1].first_z) ++ci;
+  const PlaneComp<T>& c = a.c[ci];
+  const int nxy = c.nx * c.ny, chunks = (nxy + 255) / 256, b = (int)blockIdx.x - c.first_z;
+  const int pl = b / chunks, iM = pl / c.nz, zeta = pl - iM * c.nz;
+  const int xy = (b - pl * chunks) * 256 + threadIdx.x;
+  if (xy >= nxy) return;
+  const int64_t npts = (int64_t)c.nz * nxy;
+  const T* zt = c.zt + (int64_t)zeta * (1 + 3 * a.nM) * R;
+  const T* zm = zt + (1 + 3 * iM) * R;
+  const int64_t o = (int64_t)iM * npts + (int64_t)c.bz[zeta] * nxy + xy;  // the z basis keeps all its functions
+  const int64_t out = (int64_t)pl * nxy + xy;
+  T U = 0, L = 0, D = 0, e = 0;
+  if (a.only_S) {
+#pragma unroll
+    for (int t = 0; t < R; ++t) U = fma(zt[t], c.P[o + (int64_t)t * nxy], U);
+    c.y[out] = U;
+    return;
+  }
+  const T w = c.W[out];
 #pragma unroll
   for (int t = 0; t < R; ++t) {
-    const int k = b + t;
-    if (k >= 0 && k < a.nz) {
-      const int64_t o = blk + (int64_t)k * a.nx * a.ny + xy;
-      const T p = a.P[o];
-      U = fma(a.Sz[zeta * R + t], p, U);
-      if (!only_S) {
-        Uz = fma(a.D1z[zeta * R + t], p, Uz);
-        Uzz = fma(a.D2z[zeta * R + t], p, Uzz);
-        Uxx = fma(a.Sz[zeta * R + t], a.Q[o], Uxx);
-        Uyy = fma(a.Sz[zeta * R + t], a.R[o], Uyy);
-      }
-    }
+    const T p = c.P[o + (int64_t)t * nxy];
+    U = fma(zt[t], p, U);
+    L = fma(zm[t], p, L);
+    D = fma(zt[t], c.Q[o + (int64_t)t * nxy], D);
   }
-  if (only_S) {
-    a.y[gid] = U;
-    return;
-  }
-  // pointwise coefficients folded at set-up: W = V_a + sum V^(l) + q M'(M'+1) + (J(J+1) - 2M'^2)/y^2
-  const T C = a.W[blk + pt] - a.E;
-  T out = fma(C, U, fma(a.B[blk + pt], Uz, fma(-a.A[pt], Uzz, -Uyy - Uxx)));
-  if (a.nM == 1) {
-    a.y[gid] = out;
-    return;
-  }
-  const int eta = (int)(xy % a.ny);
-  const T z = a.zp[zeta];
-  const T iy2 = a.iy2[eta];
-  const int Mp = a.M0 + iM;
-  if (iM + 1 < a.nM) {  // lambda-hat^{J,M'}/y^2 [-(1-z^2) d/dz + 2(M'+1) z] psi_{M'+1}
-    T Up = 0, Uzp = 0;
+  if (iM + 1 < a.nM) {
 #pragma unroll
-    for (int t = 0; t < R; ++t) {
-      const int k = b + t;
-      if (k >= 0 && k < a.nz) {
-        const T p = a.P[blk + npts + (int64_t)k * a.nx * a.ny + xy];
-        Up = fma(a.Sz[zeta * R + t], p, Up);
-        Uzp = fma(a.D1z[zeta * R + t], p, Uzp);
-      }
-    }
-    out += a.lamp[iM] * iy2 * (-((T)1 - z * z) * Uzp + (T)(2 * (Mp + 1)) * z * Up);
+    for (int t = 0; t < R; ++t) e = fma(zm[R + t], c.P[o + npts + (int64_t)t * nxy], e);
   }
-  if (iM >= 1) {  // lambda-hat^{J,-M'}/y^2 d/dz psi_{M'-1}
-    T Uzm = 0;
+  if (iM >= 1) {
 #pragma unroll
-    for (int t = 0; t < R; ++t) {
-      const int k = b + t;
-      if (k >= 0 && k < a.nz) Uzm = fma(a.D1z[zeta * R + t], a.P[blk - npts + (int64_t)k * a.nx * a.ny + xy], Uzm);
-    }
-    out += a.lamm[iM] * iy2 * Uzm;
+    for (int t = 0; t < R; ++t) e = fma(zm[2 * R + t], c.P[o - npts + (int64_t)t * nxy], e);
   }
-  a.y[gid] = out;
+  const int ix = xy / c.ny;
+  const T iy2 = c.iy2[xy - ix * c.ny], q = c.qx[ix] + iy2;
+  T v = fma(w - a.E, U, fma(q, L, -D));
+  if (a.nM > 1) v = fma(iy2, e, v);
+  c.y[out] = v;
 }
 
 template <typename T>
@@ -1537,7 +1715,7 @@ namespace fmi {
 
 template <typename T>
 struct ApplyTabs {
-  const T *Sx, *D2x, *Sy, *D2y, *Sz, *D1z, *D2z, *zp, *W, *A, *B, *iy2, *cval, *cw;
+  const T *Sx, *D2x, *Sy, *D2y, *zt, *qx, *W, *iy2, *cval, *cw;
 };
 
 template <typename T>
@@ -1545,66 +1723,146 @@ static ApplyTabs<T> tabs_of(const Comp& cp);
 
 template <>
 ApplyTabs<double> tabs_of<double>(const Comp& cp) {
-  return {cp.dx.S, cp.dx.D2, cp.dy.S, cp.dy.D2, cp.dz.S, cp.dz.D1, cp.dz.D2, cp.dz.pts, cp.W, cp.A, cp.B, cp.iy2,
-          cp.cpl_val, cp.cpl_w};
+  return {cp.dx.S, cp.dx.D2, cp.dy.S, cp.dy.D2, cp.zt, cp.qx, cp.W, cp.iy2, cp.cpl_val, cp.cpl_w};
 }
 
 template <>
 ApplyTabs<float> tabs_of<float>(const Comp& cp) {
-  return {cp.f32.Sx, cp.f32.D2x, cp.f32.Sy, cp.f32.D2y, cp.f32.Sz, cp.f32.D1z, cp.f32.D2z, cp.f32.zp, cp.f32.W,
-          cp.f32.A, cp.f32.B, cp.f32.iy2, cp.f32.cval, cp.f32.cw};
+  return {cp.f32.Sx, cp.f32.D2x, cp.f32.Sy, cp.f32.D2y, cp.f32.zt, cp.f32.qx, cp.f32.W, cp.f32.iy2, cp.f32.cval, cp.f32.cw};
 }
 
 template <>
 ApplyTabs<dd> tabs_of<dd>(const Comp& cp) {
-  return {cp.tdd.Sx, cp.tdd.D2x, cp.tdd.Sy, cp.tdd.D2y, cp.tdd.Sz, cp.tdd.D1z, cp.tdd.D2z, cp.tdd.zp, cp.tdd.W,
-          cp.tdd.A, cp.tdd.B, cp.tdd.iy2, cp.tdd.cval, cp.tdd.cw};
+  return {cp.tdd.Sx, cp.tdd.D2x, cp.tdd.Sy, cp.tdd.D2y, cp.tdd.zt, cp.tdd.qx, cp.tdd.W, cp.tdd.iy2, cp.tdd.cval, cp.tdd.cw};
 }
 
-// y = (H - E S) x (only_S: y = S x) with scratch planes P, Q, R, in the element type T.
-template <typename T>
-static int apply_t(fm_ctx* c, double E, const T* x, T* y, bool only_S, T* P, T* Q, T* R, bool timed) {
-  const double fscale = std::is_same<T, float>::value ? 1.0 : 1.0;
-  for (auto& cp : c->comps) {
-    const ApplyTabs<T> tb = tabs_of<T>(cp);
-    const int64_t off = cp.off;
-    constexpr int TX = 8;
-    const int rows = cp.ax.tile_rows(TX), RT = cp.r;
-    const size_t smem = (size_t)3 * rows * cp.ny * sizeof(T);
-    dim3 g1((cp.nx + TX - 1) / TX, cp.nz * c->nM);
-    {
-      const int tk_ = timed ? prof_begin(c, FM_KERNEL_APPLY_XY) : -1;
-      if (RT == 6)
-        k_apply_xy<TX, 6, T><<<g1, 256, smem, c->stream>>>(x + off, P + off, Q + off, R + off, cp.nx, cp.ny, rows,
-                                                           cp.dx.base, tb.Sx, tb.D2x, cp.dy.base, tb.Sy, tb.D2y, only_S);
-      else
-        k_apply_xy<TX, 4, T><<<g1, 256, smem, c->stream>>>(x + off, P + off, Q + off, R + off, cp.nx, cp.ny, rows,
-                                                           cp.dx.base, tb.Sx, tb.D2x, cp.dy.base, tb.Sy, tb.D2y, only_S);
-      prof_end(c, tk_, fscale * cp.npts * c->nM * RT * (only_S ? 4.0 : 10.0),
-               (double)cp.npts * c->nM * (only_S ? 2.0 : 4.0) * sizeof(T));
-    }
-    c->launches++;
-    ZPassArgs<T> a;
-    a.P = P + off; a.Q = Q + off; a.R = R + off; a.y = y + off; a.W = tb.W; a.A = tb.A; a.B = tb.B; a.iy2 = tb.iy2;
-    a.bz = cp.dz.base; a.Sz = tb.Sz; a.D1z = tb.D1z; a.D2z = tb.D2z; a.zp = tb.zp;
-    a.nx = cp.nx; a.ny = cp.ny; a.nz = cp.nz; a.nM = c->nM; a.M0 = c->M0; a.J = c->sys.J; a.E = (T)E;
-    for (int i = 0; i < kMaxM; ++i) a.lamp[i] = a.lamm[i] = (T)0;
-    for (int iM = 0; iM < c->nM; ++iM) {
-      const int Mp = c->Mps[iM], J = c->sys.J;
-      const double vp = (double)(J * (J + 1) - Mp * (Mp + 1)), vm = (double)(J * (J + 1) - Mp * (Mp - 1));
-      a.lamp[iM] = (T)((vp > 0 ? sqrt(vp) : 0.0) * sqrt(Mp == 0 ? 2.0 : 1.0));
-      a.lamm[iM] = (T)((vm > 0 ? sqrt(vm) : 0.0) * sqrt(Mp == 1 ? 2.0 : 1.0));
-    }
-    const int64_t tot = cp.npts * c->nM;
-    {
-      const int tk_ = timed ? prof_begin(c, FM_KERNEL_APPLY_Z) : -1;
-      if (RT == 6) k_apply_z<6, T><<<(unsigned)((tot + 255) / 256), 256, 0, c->stream>>>(a, only_S);
-      else k_apply_z<4, T><<<(unsigned)((tot + 255) / 256), 256, 0, c->stream>>>(a, only_S);
-      prof_end(c, tk_, (double)tot * (only_S ? 2.0 * RT : (10.0 + (c->nM > 1 ? 8.0 * RT : 0.0) + 10.0 * RT)),
-               (double)tot * (only_S ? 2.0 : 7.0) * sizeof(T));
-    }
-    c->launches++;
+// largest n_M of k_apply_local per r: its register planes are 2 r n_M values
+constexpr int kLocalMaxM4 = 5, kLocalMaxM6 = 3;
+
+// The local part of the operator on every component in float32, one launch (k_apply_local).
+static int apply_local32(fm_ctx* c, double E, const float* x, float* y, bool only_S, bool timed) {
+  LocalArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.ncomp = (int)c->comps.size();
+  a.E = (float)E;
+  a.only_S = only_S ? 1 : 0;
+  const int r = c->comps[0].r, q = c->comps[0].az.q;
+  int tiles = 0, nintmax = 1, smem_elems = 0;
+  double fl = 0.0, by = 0.0;
+  for (int k = 0; k < a.ncomp; ++k) {
+    const Comp& cp = c->comps[k];
+    const ApplyTabs<float> tb = tabs_of<float>(cp);
+    LocalComp& f = a.c[k];
+    f.x = x + cp.off; f.y = y + cp.off; f.W = tb.W; f.Sx = tb.Sx; f.D2x = tb.D2x; f.Sy = tb.Sy; f.D2y = tb.D2y;
+    f.zt = tb.zt; f.qx = tb.qx; f.iy2 = tb.iy2; f.bx = cp.dx.base; f.by = cp.dy.base; f.zf = cp.zf;
+    f.nx = cp.nx; f.ny = cp.ny; f.nz = cp.nz; f.rows = cp.ax.tile_rows(kLX); f.cols = cp.ay.tile_rows(kLY);
+    f.tiles_x = (cp.nx + kLX - 1) / kLX; f.tiles_y = (cp.ny + kLY - 1) / kLY;
+    f.nint = cp.az.nint; f.q = q;
+    tiles += f.tiles_x * f.tiles_y;
+    nintmax = std::max(nintmax, f.nint);
+    smem_elems = std::max(smem_elems, 2 * r * (kLX + kLY) + q * c->nM * f.rows * (2 * (f.cols + 1) + 2 * kLY));
+    const double tot = (double)cp.npts * c->nM;
+    fl += tot * (only_S ? 6.0 * r : (c->nM > 1 ? 20.0 : 16.0) * r + 6.0);
+    by += tot * (only_S ? 2.0 : 3.0) * sizeof(float);
   }
+  // z chunks: a CTA of n intervals walks q n + r - q planes; the split with the fewest planes on the SM that gets the
+  // most CTAs, counting at least four (fewer leave the latency of a plane uncovered)
+  int ipc = 1;
+  double cost = 1e300;
+  for (int n = 1; n <= nintmax; ++n) {
+    const int per_cta = (nintmax + n - 1) / n;
+    const int ctas = tiles * ((nintmax + per_cta - 1) / per_cta);
+    const double cst = std::max(4, (ctas + 151) / 152) * (double)(q * per_cta + r - q);
+    if (cst < cost) {
+      cost = cst;
+      ipc = per_cta;
+    }
+  }
+  int grid = 0;
+  for (int k = 0; k < a.ncomp; ++k) {
+    LocalComp& f = a.c[k];
+    f.ipc = std::min(ipc, f.nint);
+    f.first = grid;
+    grid += f.tiles_x * f.tiles_y * ((f.nint + f.ipc - 1) / f.ipc);
+  }
+  const size_t smem = (size_t)smem_elems * sizeof(float);
+  const int tk_ = timed ? prof_begin(c, FM_KERNEL_APPLY_XY) : -1;
+  switch ((r == 6 ? 16 : 0) + c->nM) {
+    case 1: k_apply_local<4, 1><<<grid, kLThreads, smem, c->stream>>>(a); break;
+    case 2: k_apply_local<4, 2><<<grid, kLThreads, smem, c->stream>>>(a); break;
+    case 3: k_apply_local<4, 3><<<grid, kLThreads, smem, c->stream>>>(a); break;
+    case 4: k_apply_local<4, 4><<<grid, kLThreads, smem, c->stream>>>(a); break;
+    case 5: k_apply_local<4, 5><<<grid, kLThreads, smem, c->stream>>>(a); break;
+    case 17: k_apply_local<6, 1><<<grid, kLThreads, smem, c->stream>>>(a); break;
+    case 18: k_apply_local<6, 2><<<grid, kLThreads, smem, c->stream>>>(a); break;
+    case 19: k_apply_local<6, 3><<<grid, kLThreads, smem, c->stream>>>(a); break;
+    default: return FM_ERR_ARG;
+  }
+  prof_end(c, tk_, fl, by);
+  c->launches++;
+  FM_CUDA(cudaGetLastError());
+  return FM_OK;
+}
+
+// The local part of the operator in two passes (scratch planes P and Q), every component in each launch.
+template <typename T>
+static int apply_planes(fm_ctx* c, double E, const T* x, T* y, bool only_S, T* P, T* Q, bool timed) {
+  PlaneArgs<T> a;
+  std::memset(&a, 0, sizeof(a));
+  a.ncomp = (int)c->comps.size();
+  a.nM = c->nM;
+  a.E = (T)E;
+  a.only_S = only_S ? 1 : 0;
+  const int r = c->comps[0].r;
+  int64_t gxy = 0, gz = 0;
+  size_t elems = 0;
+  double tot = 0.0;
+  for (int k = 0; k < a.ncomp; ++k) {
+    const Comp& cp = c->comps[k];
+    const ApplyTabs<T> tb = tabs_of<T>(cp);
+    PlaneComp<T>& f = a.c[k];
+    f.x = x + cp.off; f.P = P + cp.off; f.Q = Q + cp.off; f.y = y + cp.off; f.W = tb.W; f.Sx = tb.Sx; f.D2x = tb.D2x;
+    f.Sy = tb.Sy; f.D2y = tb.D2y; f.zt = tb.zt; f.qx = tb.qx; f.iy2 = tb.iy2;
+    f.bx = cp.dx.base; f.by = cp.dy.base; f.bz = cp.dz.base;
+    f.nx = cp.nx; f.ny = cp.ny; f.nz = cp.nz; f.rows = cp.ax.tile_rows(kPX); f.cols = cp.ay.tile_rows(kPY);
+    f.tiles_x = (cp.nx + kPX - 1) / kPX; f.tiles_y = (cp.ny + kPY - 1) / kPY;
+    f.first_xy = (int)gxy;
+    f.first_z = (int)gz;
+    const int64_t planes = (int64_t)c->nM * cp.nz;
+    gxy += planes * f.tiles_x * f.tiles_y;
+    gz += planes * (((int64_t)cp.nx * cp.ny + 255) / 256);
+    elems = std::max(elems, (size_t)f.rows * (f.cols + 1 + 2 * kPY));
+    tot += (double)cp.npts * c->nM;
+  }
+  if (gxy > 0x7FFFFFFF || gz > 0x7FFFFFFF) return FM_ERR_ARG;
+  {
+    const int tk_ = timed ? prof_begin(c, FM_KERNEL_APPLY_XY) : -1;
+    if (r == 6) k_apply_xy<6, T><<<(unsigned)gxy, 256, elems * sizeof(T), c->stream>>>(a);
+    else k_apply_xy<4, T><<<(unsigned)gxy, 256, elems * sizeof(T), c->stream>>>(a);
+    prof_end(c, tk_, tot * r * (only_S ? 4.0 : 10.0), tot * (only_S ? 2.0 : 3.0) * sizeof(T));
+  }
+  {
+    const int tk_ = timed ? prof_begin(c, FM_KERNEL_APPLY_Z) : -1;
+    if (r == 6) k_apply_z<6, T><<<(unsigned)gz, 256, 0, c->stream>>>(a);
+    else k_apply_z<4, T><<<(unsigned)gz, 256, 0, c->stream>>>(a);
+    prof_end(c, tk_, tot * (only_S ? 2.0 * r : (c->nM > 1 ? 10.0 : 6.0) * r + 6.0),
+             tot * (only_S ? 2.0 : 4.0) * sizeof(T));
+  }
+  c->launches += 2;
+  FM_CUDA(cudaGetLastError());
+  return FM_OK;
+}
+
+// y = (H - E S) x (only_S: y = S x) in the element type T; scratch planes P and Q for the two-pass local form.
+template <typename T>
+static int apply_t(fm_ctx* c, double E, const T* x, T* y, bool only_S, T* P, T* Q, bool timed) {
+  int rc;
+  bool one_pass = false;
+  if constexpr (std::is_same<T, float>::value) {
+    one_pass = c->nM <= (c->comps[0].r == 6 ? kLocalMaxM6 : kLocalMaxM4);
+    if (one_pass && (rc = apply_local32(c, E, x, y, only_S, timed))) return rc;
+  }
+  if (!one_pass && (rc = apply_planes<T>(c, E, x, y, only_S, P, Q, timed))) return rc;
   const bool staged = std::is_same<T, float>::value && c->ystage32 != nullptr;
   if (!only_S && staged) {  // float32: regroup every source component's y coefficients by y interval
     for (auto& cp : c->comps) {
@@ -1668,18 +1926,18 @@ static int apply_t(fm_ctx* c, double E, const T* x, T* y, bool only_S, T* P, T* 
 }
 
 int launch_apply(fm_ctx* c, double E, const double* x, double* y, bool only_S) {
-  return apply_t<double>(c, E, x, y, only_S, c->P, c->Q, c->R, true);
+  return apply_t<double>(c, E, x, y, only_S, c->P, c->Q, true);
 }
 
 int launch_apply32(fm_ctx* c, double E, const float* x, float* y, bool only_S) {
-  return apply_t<float>(c, E, x, y, only_S, c->P32, c->Q32, c->R32, true);
+  return apply_t<float>(c, E, x, y, only_S, c->P32, c->Q32, true);
 }
 
 // The operator apply with caller-chosen scratch planes (used by the entry point that allocates
 // nothing, whose planes live in a fixed device array).  Same kernels and launch shapes as
 // launch_apply; no per-kernel timing.
-int launch_apply_scratch(fm_ctx* c, double E, const double* x, double* y, double* P, double* Q, double* R) {
-  return apply_t<double>(c, E, x, y, false, P, Q, R, false);
+int launch_apply_scratch(fm_ctx* c, double E, const double* x, double* y, double* P, double* Q) {
+  return apply_t<double>(c, E, x, y, false, P, Q, false);
 }
 
 // Banded y solves (Eq. prec-2 y stage with the M' chain) of the given components in one launch,
@@ -2284,7 +2542,7 @@ int launch_apply_dd(fm_ctx* c, double E, const dd* x, dd* y, bool only_S) {
   // the float64 scratch planes, read as dd (the same 8 bytes per element; the float64 and dd applies never
   // overlap)
   return apply_t<dd>(c, E, x, y, only_S, reinterpret_cast<dd*>(c->P), reinterpret_cast<dd*>(c->Q),
-                     reinterpret_cast<dd*>(c->R), true);
+                     true);
 }
 
 int launch_precond_dd(fm_ctx* c, const dd* x, dd* y) {
@@ -2417,12 +2675,12 @@ int* tc_flag_slot(fm_ctx* c) { return reinterpret_cast<int*>(c->gsd + kGsFlag); 
 
 int kernels_init(fm_ctx* c) {
   (void)c;
-  FM_CUDA(cudaFuncSetAttribute(k_apply_xy<8, 4, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  FM_CUDA(cudaFuncSetAttribute(k_apply_xy<8, 4, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  FM_CUDA(cudaFuncSetAttribute(k_apply_xy<8, 6, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  FM_CUDA(cudaFuncSetAttribute(k_apply_xy<8, 6, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  FM_CUDA(cudaFuncSetAttribute(k_apply_xy<8, 4, dd>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  FM_CUDA(cudaFuncSetAttribute(k_apply_xy<8, 6, dd>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  const int most = 200 * 1024;
+  FM_CUDA(cudaFuncSetAttribute(k_apply_local<4, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+  FM_CUDA(cudaFuncSetAttribute(k_apply_local<4, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+  FM_CUDA(cudaFuncSetAttribute(k_apply_local<6, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+  FM_CUDA(cudaFuncSetAttribute(k_apply_local<6, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
+  FM_CUDA(cudaFuncSetAttribute(k_apply_local<6, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
   FM_CUDA(cudaFuncSetAttribute(k_zmix<double, double, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   FM_CUDA(cudaFuncSetAttribute(k_zmix<double, float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   FM_CUDA(cudaFuncSetAttribute(k_zmix<float, double, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));

@@ -77,5 +77,5 @@ extern "C" int fm_apply_noalloc(fm_ctx* ctx, double E, const double* x, double* 
   const int64_t N = ctx->N;
   // every scratch element the kernels read is written earlier in the same call, so the contents
   // left by a previous call need no clearing
-  return fmi::launch_apply_scratch(ctx, E, x, y, s, s + N, s + 2 * N);
+  return fmi::launch_apply_scratch(ctx, E, x, y, s, s + N);
 }

@@ -544,8 +544,26 @@ int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
     if ((rc = upload_axis(c, cp.az, cp.dz))) return rc;
     // pointwise coefficients of Eq. FM-pre: the left-hand potential V_a(x) + sum_{b != a} V^(l)_b(x_b, y_b)
     // folded with the M'-dependent diagonal terms, and the coefficients of the z derivatives
-    std::vector<double> W((size_t)nM * cp.npts), Atab((size_t)cp.npts), Btab((size_t)nM * cp.npts), iy2(cp.ny);
+    std::vector<double> W((size_t)nM * cp.npts), iy2(cp.ny), qx(cp.nx), zt((size_t)cp.nz * (1 + 3 * nM) * cp.r);
     for (int j = 0; j < cp.ny; ++j) iy2[j] = 1.0 / (cp.ay.pts[j] * cp.ay.pts[j]);
+    for (int i = 0; i < cp.nx; ++i) qx[i] = 1.0 / (cp.ax.pts[i] * cp.ax.pts[i]);
+    std::vector<int> zf(cp.az.nint + 1, cp.nz);  // the z basis keeps all its functions: base = q m in interval m
+    for (int k = cp.nz - 1; k >= 0; --k) zf[cp.az.base[k] / cp.az.q] = k;
+    for (int k = 0; k < cp.nz; ++k) {
+      const double z = cp.az.pts[k];
+      double* t = &zt[(size_t)k * (1 + 3 * nM) * cp.r];
+      for (int e = 0; e < cp.r; ++e) {
+        const double Sz = cp.az.S[k * cp.r + e], D1 = cp.az.D1[k * cp.r + e], D2 = cp.az.D2[k * cp.r + e];
+        t[e] = Sz;
+        for (int iM = 0; iM < nM; ++iM) {
+          const int Mp = c->Mps[iM];
+          double* tm3 = t + (1 + 3 * iM) * cp.r;
+          tm3[e] = 2.0 * (Mp + 1) * z * D1 - (1.0 - z * z) * D2;
+          tm3[cp.r + e] = lam_hat_plus(J, Mp) * (2.0 * (Mp + 1) * z * Sz - (1.0 - z * z) * D1);
+          tm3[2 * cp.r + e] = lam_hat_minus(J, Mp) * D1;
+        }
+      }
+    }
     std::vector<int> bad_plane(cp.nz, 0);
     const Comp* cq = &cp;
     parallel_for(cp.nz, [&](int k) {  // one z plane per task
@@ -565,11 +583,9 @@ int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
           if (!std::isfinite(tot)) bad_plane[k] = 1;
           const size_t pt = ((size_t)k * cq->nx + i) * cq->ny + j;
           const double q = 1.0 / (x * x) + iy2[j];
-          Atab[pt] = q * (1.0 - z * z);
           for (int iM = 0; iM < nM; ++iM) {
             const int Mp = c->Mps[iM];
             W[(size_t)iM * cq->npts + pt] = tot + q * Mp * (Mp + 1.0) + (J * (J + 1.0) - 2.0 * Mp * Mp) * iy2[j];
-            Btab[(size_t)iM * cq->npts + pt] = 2.0 * (Mp + 1) * z * q;
           }
         }
     });
@@ -577,8 +593,9 @@ int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
       if (b) return FM_ERR_NUMERIC;
     tm.mark("potential tables");
     if ((rc = upload(c, (void**)&cp.W, W.data(), W.size() * sizeof(double)))) return rc;
-    if ((rc = upload(c, (void**)&cp.A, Atab.data(), Atab.size() * sizeof(double)))) return rc;
-    if ((rc = upload(c, (void**)&cp.B, Btab.data(), Btab.size() * sizeof(double)))) return rc;
+    if ((rc = upload(c, (void**)&cp.zt, zt.data(), zt.size() * sizeof(double)))) return rc;
+    if ((rc = upload(c, (void**)&cp.qx, qx.data(), qx.size() * sizeof(double)))) return rc;
+    if ((rc = upload(c, (void**)&cp.zf, zf.data(), zf.size() * sizeof(int)))) return rc;
     if ((rc = upload(c, (void**)&cp.iy2, iy2.data(), iy2.size() * sizeof(double)))) return rc;
     {  // float32 copies for the mixed-precision inner solves
       auto up32 = [&](float** dst, const std::vector<double>& v) {
@@ -586,9 +603,8 @@ int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
         return upload(c, (void**)dst, f.data(), f.size() * sizeof(float));
       };
       if ((rc = up32(&cp.f32.Sx, cp.ax.S)) || (rc = up32(&cp.f32.D2x, cp.ax.D2)) || (rc = up32(&cp.f32.Sy, cp.ay.S)) ||
-          (rc = up32(&cp.f32.D2y, cp.ay.D2)) || (rc = up32(&cp.f32.Sz, cp.az.S)) || (rc = up32(&cp.f32.D1z, cp.az.D1)) ||
-          (rc = up32(&cp.f32.D2z, cp.az.D2)) || (rc = up32(&cp.f32.zp, cp.az.pts)) || (rc = up32(&cp.f32.W, W)) ||
-          (rc = up32(&cp.f32.A, Atab)) || (rc = up32(&cp.f32.B, Btab)) || (rc = up32(&cp.f32.iy2, iy2)))
+          (rc = up32(&cp.f32.D2y, cp.ay.D2)) || (rc = up32(&cp.f32.zt, zt)) || (rc = up32(&cp.f32.qx, qx)) ||
+          (rc = up32(&cp.f32.W, W)) || (rc = up32(&cp.f32.iy2, iy2)))
         return rc;
     }
     if (c->use_dd) {  // double-float copies for the double-float inner solves
@@ -597,9 +613,8 @@ int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
         return upload(c, (void**)dst, f.data(), f.size() * sizeof(dd));
       };
       if ((rc = updd(&cp.tdd.Sx, cp.ax.S)) || (rc = updd(&cp.tdd.D2x, cp.ax.D2)) || (rc = updd(&cp.tdd.Sy, cp.ay.S)) ||
-          (rc = updd(&cp.tdd.D2y, cp.ay.D2)) || (rc = updd(&cp.tdd.Sz, cp.az.S)) || (rc = updd(&cp.tdd.D1z, cp.az.D1)) ||
-          (rc = updd(&cp.tdd.D2z, cp.az.D2)) || (rc = updd(&cp.tdd.zp, cp.az.pts)) || (rc = updd(&cp.tdd.W, W)) ||
-          (rc = updd(&cp.tdd.A, Atab)) || (rc = updd(&cp.tdd.B, Btab)) || (rc = updd(&cp.tdd.iy2, iy2)))
+          (rc = updd(&cp.tdd.D2y, cp.ay.D2)) || (rc = updd(&cp.tdd.zt, zt)) || (rc = updd(&cp.tdd.qx, qx)) ||
+          (rc = updd(&cp.tdd.W, W)) || (rc = updd(&cp.tdd.iy2, iy2)))
         return rc;
     }
 
@@ -876,8 +891,8 @@ int estimate_bytes(const fm_system* S, const fm_grid* grids, int n_grids, const 
     const double nx = ax.n, ny = ay.n, nz = az.n, npts = nx * ny * nz;
     N += (int64_t)(npts * nM);
     bytes += (nx + ny + nz) * (4 + 3 * R * 12 + 8) * 1.5;              // tap tables (float64 + float32)
-    bytes += (2.0 * nM + 1.0) * npts * 12.0 + ny * 12.0;                 // W, B per M'; A; iy2 (+ float32)
-    dd_tables += (nx + ny + nz) * 3 * R * 8 + (2.0 * nM + 1.0) * npts * 8.0;
+    bytes += nM * npts * 12.0 + (nx + ny) * 12.0 + nz * (1.0 + 3.0 * nM) * R * 12.0;  // W; 1/x^2, 1/y^2; z taps (+ float32)
+    dd_tables += (nx + ny + nz) * 3 * R * 8 + nM * npts * 8.0 + nz * (1.0 + 3.0 * nM) * R * 8.0;
     if (split->mode != FM_SPLIT_SCHRODINGER) {                           // coupling geometry
       double act = 0.0;
       for (int i = 0; i < ax.n; ++i)
@@ -914,9 +929,9 @@ int estimate_bytes(const fm_system* S, const fm_grid* grids, int n_grids, const 
   const double m = o->restart_m, ncv = o->ncv, n = (double)N;
   if (o->precision == FM_PREC_MIXED && o->mixed_scheme == 2)
     bytes += dd_tables + n * 8.0 * ((m + 1) + m + 4);                  // double-float tables and Krylov vectors
-  bytes += n * 8.0 * (5 + 2 + 3 + 16) + n * 4.0 * 2;                    // apply scratch, stage buffers, tuning
+  bytes += n * 8.0 * (5 + 2 + 2 + 16) + n * 4.0 * 2;                    // apply scratch, stage buffers, tuning
   bytes += n * 8.0 * ((m + 1) + std::max(m, ncv) + (ncv + 1));          // FGMRES and Arnoldi bases
-  if (o->precision == FM_PREC_MIXED) bytes += n * 4.0 * ((m + 1) + m + 7 + 2.5);  // + y-interval sources
+  if (o->precision == FM_PREC_MIXED) bytes += n * 4.0 * ((m + 1) + m + 6 + 2.5);  // + y-interval sources
   bytes += (4.0 * 152 * 256 + 8192 + 4096) * 8.0;
   *out = (int64_t)bytes;
   return FM_OK;
