@@ -99,9 +99,10 @@ struct Comp {
   double* iy2 = nullptr;         // [ny] 1/y^2
   // coupling tables: n_act active points, per (source s): taps and weights
   int n_act = 0;
+  bool cpl_mirror = false;       // source 1 at z is source 0 at -z: one set of taps serves both
   int* act_pt = nullptr;         // [n_act] point index (k*nx + i)*ny + j
-  int* cpl_base = nullptr;       // [ns][3][n_act]  (z, x, y tap bases)
-  double* cpl_val = nullptr;     // [ns][3 r][n_act] (Sz[r], Sx[r], Sy[r])
+  int* cpl_base = nullptr;       // [ns, or 1 when mirrored][3][n_act]  (z, x, y tap bases; z base -1: outside the box)
+  double* cpl_val = nullptr;     // [ns or 1][3 r][n_act] (Sz[r], Sx[r], Sy[r])
   double* cpl_w = nullptr;       // [ns][nM*nM][n_act] weight of (M', M'')
   // preconditioner, E-independent
   double* Wz = nullptr;          // [nM][nz][nz]

@@ -357,60 +357,108 @@ __global__ void __launch_bounds__(256) k_apply_z(const __grid_constant__ PlaneAr
   c.y[out] = v;
 }
 
+// ---------------------------------------------------------------------------
+// V^(s) coupling (Eqs. r-form, s-rot): every active collocation point adds the other components' expansions at its
+// rotated position, r x r x r taps per source and M''.  One launch serves every component; bound by the FP64 pipe
+// (r^3 + r^2 + r multiply-adds per point, source and M''), in float32 by L1.
+//   * A (point, source) pair whose rotated position lies outside the source's box (z base -1) is passed over: the
+//     expansion is zero there.  With boxes of different sizes most pairs of the wide component are outside.
+//   * With an identical pair both sources of the third component are the same expansion, and on a z grid symmetric
+//     about 0 source 2 at (x, y, z) is source 1 at (x, y, -z) (the rotations of an exchanged pair differ in the
+//     sign of s alone).  Its points are then taken in pairs (zeta, n_z - 1 - zeta) that share two evaluations
+//     instead of four.
+// He L = 0 96 x 96 x 24: 463 -> 342 us (0.95 of the FP64 pipe); J = 2..4 on mid-size grids 1.4 .. 2.1x (the sums over
+// M' in registers: their count is a template argument); He J = 10 and unequal boxes gain most from the skipped pairs.
+// ---------------------------------------------------------------------------
 template <typename T>
-struct CouplingArgs {
-  const T* x;           // full input vector
-  T* y;                 // full output vector (accumulated)
-  int64_t row_off;      // offset of the target component
-  int64_t npts;         // points per M' block of the target component
-  int n_act;
+struct CplSource {
+  const int* base;      // [3][n_act] (z, x, y) tap bases
+  const T* val;         // [3 R][n_act]
+  const T* w;           // [nM * nM][n_act]
+  const T* src;         // the source component's coefficients
+  const T* stage;       // float32: y coefficients regrouped by y interval, [nM][nz][nx][nint_y][R]
+  int64_t npts;
+  int nx, ny, nz, nint;
+};
+template <typename T>
+struct CplComp {
+  CplSource<T> s[3];
+  T* y;
   const int* act_pt;
-  int ns;
-  const int* base[3];   // per source: [3][n_act]
-  const T* val[3];      // per source: [12][n_act]
-  const T* w[3];        // per source: [nM*nM][n_act]
-  int64_t src_off[3];
-  int64_t src_npts[3];
-  int snx[3], sny[3], snz[3];
-  int nM;
-  // staged source (float32 path): per source, the y coefficients regrouped by y interval
-  const T* stage[3];    // [nM][nz][nx][nint_y][R] of the source component
-  int snint[3];         // y intervals of the source
-  int sdir;             // 1: Dirichlet y basis (base = q m - 1), so interval m = (base + 1) / q
-  int sq;               // functions per node
+  int64_t npts;
+  int n_act, ns;
+  int mirror, nz, nxy;  // mirrored pairs of sources 0 and 1: z points, active points per z plane
+  int first;            // first block
+};
+template <typename T>
+struct CplArgs {
+  CplComp<T> c[3];
+  int ncomp, nM;
+  int sdir, sq;         // float32: interval of a y base = (base + sdir) / sq
 };
 
-// V^(s) coupling: one thread per active collocation point of a component; R x R x R taps of the source
-// expansion at the rotated point.
-template <int R, typename T>
-__global__ void __launch_bounds__(128) k_apply_coupling(CouplingArgs<T> a) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= a.n_act) return;
-  T acc[kMaxM];
+// the source's expansion of every M'' at point p; false outside its box
+template <int R, int NMC, typename T>
+__device__ __forceinline__ bool cpl_eval(const CplSource<T>& s, int p, int n_act, int nM, int sdir, int sq, T* E) {
+  const int bz = s.base[p];
+  if (bz < 0) return false;
+  const int bx = s.base[n_act + p], by = s.base[2 * n_act + p];
+  T vz[R], vx[R], vy[R];
+  int ix[R];
 #pragma unroll
-  for (int m = 0; m < kMaxM; ++m) acc[m] = (T)0;
-  for (int s = 0; s < a.ns; ++s) {
-    const int bz = a.base[s][p], bx = a.base[s][a.n_act + p], by = a.base[s][2 * a.n_act + p];
-    T vz[R], vx[R], vy[R];
-    int iz[R], ix[R], iy[R];
+  for (int t = 0; t < R; ++t) {
+    vz[t] = s.val[(0 * R + t) * (int64_t)n_act + p];
+    vx[t] = s.val[(1 * R + t) * (int64_t)n_act + p];
+    vy[t] = s.val[(2 * R + t) * (int64_t)n_act + p];
+    ix[t] = min(max(bx + t, 0), s.nx - 1);
+  }
+  if constexpr (std::is_same<T, float>::value) {
+    // regrouped by y interval: a source row's R taps are one aligned vector load
+    const int my = min(max((by + sdir) / sq, 0), s.nint - 1);
 #pragma unroll
-    for (int t = 0; t < R; ++t) {
-      vz[t] = a.val[s][(0 * R + t) * (int64_t)a.n_act + p];
-      vx[t] = a.val[s][(1 * R + t) * (int64_t)a.n_act + p];
-      vy[t] = a.val[s][(2 * R + t) * (int64_t)a.n_act + p];
-      iz[t] = min(max(bz + t, 0), a.snz[s] - 1);
-      ix[t] = min(max(bx + t, 0), a.snx[s] - 1);
-      iy[t] = min(max(by + t, 0), a.sny[s] - 1);
+    for (int jM = 0; jM < (NMC ? NMC : kMaxM); ++jM) {
+      if (!NMC && jM >= nM) break;
+      const float* tb = s.stage + (int64_t)jM * s.nz * s.nx * s.nint * R;
+      float sz = 0.f;
+#pragma unroll
+      for (int tz = 0; tz < R; ++tz) {
+        const int64_t rz = (int64_t)(bz + tz) * s.nx;
+        float sx = 0.f;
+#pragma unroll
+        for (int tx = 0; tx < R; ++tx) {
+          const float* row = tb + ((rz + ix[tx]) * s.nint + my) * R;
+          float sy = 0.f;
+          if constexpr (R == 4) {
+            const float4 c4 = __ldg(reinterpret_cast<const float4*>(row));
+            sy = fmaf(vy[3], c4.w, fmaf(vy[2], c4.z, fmaf(vy[1], c4.y, vy[0] * c4.x)));
+          } else {
+#pragma unroll
+            for (int t = 0; t < R; t += 2) {
+              const float2 c2 = __ldg(reinterpret_cast<const float2*>(row + t));
+              sy = fmaf(vy[t + 1], c2.y, fmaf(vy[t], c2.x, sy));
+            }
+          }
+          sx = fmaf(vx[tx], sy, sx);
+        }
+        sz = fmaf(vz[tz], sx, sz);
+      }
+      E[jM] = sz;
     }
-    for (int jM = 0; jM < a.nM; ++jM) {
-      const T* cb = a.x + a.src_off[s] + (int64_t)jM * a.src_npts[s];
+  } else {
+    int iy[R];
+#pragma unroll
+    for (int t = 0; t < R; ++t) iy[t] = min(max(by + t, 0), s.ny - 1);
+#pragma unroll
+    for (int jM = 0; jM < (NMC ? NMC : kMaxM); ++jM) {
+      if (!NMC && jM >= nM) break;
+      const T* cb = s.src + (int64_t)jM * s.npts;
       T sz = 0;
 #pragma unroll
       for (int tz = 0; tz < R; ++tz) {
         T sx = 0;
 #pragma unroll
         for (int tx = 0; tx < R; ++tx) {
-          const T* row = cb + ((int64_t)iz[tz] * a.snx[s] + ix[tx]) * a.sny[s];
+          const T* row = cb + ((int64_t)(bz + tz) * s.nx + ix[tx]) * s.ny;
           T sy = vy[0] * row[iy[0]];
 #pragma unroll
           for (int ty = 1; ty < R; ++ty) sy = fma(vy[ty], row[iy[ty]], sy);
@@ -418,98 +466,111 @@ __global__ void __launch_bounds__(128) k_apply_coupling(CouplingArgs<T> a) {
         }
         sz = fma(vz[tz], sx, sz);
       }
-      for (int iM = 0; iM < a.nM; ++iM)
-        acc[iM] = fma(a.w[s][(int64_t)(iM * a.nM + jM) * a.n_act + p], sz, acc[iM]);
+      E[jM] = sz;
     }
   }
-  const int pt = a.act_pt[p];
-  for (int iM = 0; iM < a.nM; ++iM) a.y[a.row_off + (int64_t)iM * a.npts + pt] += acc[iM];
+  return true;
+}
+
+// acc[iM] += sum_jM w[iM][jM](p) E[jM]
+template <int NMC, typename T>
+__device__ __forceinline__ void cpl_add(const T* w, int p, int n_act, int nM, const T* E, T* acc) {
+#pragma unroll
+  for (int iM = 0; iM < (NMC ? NMC : kMaxM); ++iM) {
+    if (!NMC && iM >= nM) break;
+#pragma unroll
+    for (int jM = 0; jM < (NMC ? NMC : kMaxM); ++jM) {
+      if (!NMC && jM >= nM) break;
+      acc[iM] = fma(w[(int64_t)(iM * nM + jM) * n_act + p], E[jM], acc[iM]);
+    }
+  }
+}
+
+template <int R, int NMC, typename T>
+__global__ void __launch_bounds__(128) k_apply_coupling(const __grid_constant__ CplArgs<T> a) {
+  constexpr int NA = NMC ? NMC : kMaxM;
+  int ci = 0;
+  while (ci + 1 < a.ncomp && (int)blockIdx.x >= a.c[ci + 1].first) ++ci;
+  const CplComp<T>& c = a.c[ci];
+  const int item = ((int)blockIdx.x - c.first) * blockDim.x + threadIdx.x;
+  const int nM = NMC ? NMC : a.nM;
+  T acc[NA], E[NA];
+#pragma unroll
+  for (int m = 0; m < NA; ++m) acc[m] = (T)0;
+  if (!c.mirror) {
+    if (item >= c.n_act) return;
+    bool any = false;
+    for (int s = 0; s < c.ns; ++s) {
+      if (!cpl_eval<R, NMC, T>(c.s[s], item, c.n_act, nM, a.sdir, a.sq, E)) continue;
+      cpl_add<NMC, T>(c.s[s].w, item, c.n_act, nM, E, acc);
+      any = true;
+    }
+    if (!any) return;
+    T* y = c.y + c.act_pt[item];
+#pragma unroll
+    for (int iM = 0; iM < NA; ++iM)
+      if (iM < nM) y[(int64_t)iM * c.npts] += acc[iM];
+    return;
+  }
+  // planes zeta and n_z - 1 - zeta
+  const int zeta = item / c.nxy;
+  if (2 * zeta >= c.nz) return;
+  const int p = item, pm = item + (c.nz - 1 - 2 * zeta) * c.nxy;
+  T accm[NA];
+#pragma unroll
+  for (int m = 0; m < NA; ++m) accm[m] = (T)0;
+  bool any = false;
+  if (cpl_eval<R, NMC, T>(c.s[0], p, c.n_act, nM, a.sdir, a.sq, E)) {
+    cpl_add<NMC, T>(c.s[0].w, p, c.n_act, nM, E, acc);
+    cpl_add<NMC, T>(c.s[1].w, pm, c.n_act, nM, E, accm);
+    any = true;
+  }
+  if (cpl_eval<R, NMC, T>(c.s[0], pm, c.n_act, nM, a.sdir, a.sq, E)) {
+    cpl_add<NMC, T>(c.s[0].w, pm, c.n_act, nM, E, accm);
+    cpl_add<NMC, T>(c.s[1].w, p, c.n_act, nM, E, acc);
+    any = true;
+  }
+  if (!any) return;
+  T *y = c.y + c.act_pt[p], *ym = c.y + c.act_pt[pm];
+#pragma unroll
+  for (int iM = 0; iM < NA; ++iM)
+    if (iM < nM) {
+      y[(int64_t)iM * c.npts] += acc[iM];
+      ym[(int64_t)iM * c.npts] += accm[iM];
+    }
 }
 
 // The y coefficients of a component regrouped by y interval: T[row][m][t] = c[row][q m - d + t] for every
 // (M', k, i) row, interval m and tap t (0 outside the basis), so that the R taps a point of interval m
-// reads are contiguous and aligned.  One thread per (row, interval).
+// reads are contiguous and aligned.  One thread per (row, interval); blockIdx.y = component.
+struct StageArgs {
+  const float* c[3];
+  float* T[3];
+  int64_t rows[3];
+  int ny[3], nint[3];
+  int q, d;
+};
 template <int R>
-__global__ void __launch_bounds__(256) k_stage_ytaps(const float* __restrict__ c, float* __restrict__ T, int64_t rows,
-                                                     int ny, int nint, int q, int d) {
+__global__ void __launch_bounds__(256) k_stage_ytaps(const StageArgs a) {
+  const int cq = blockIdx.y, nint = a.nint[cq], ny = a.ny[cq];
   const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= rows * nint) return;
+  if (gid >= a.rows[cq] * nint) return;
   const int64_t row = gid / nint;
   const int m = (int)(gid - row * nint);
-  const float* cr = c + row * ny;
+  const float* cr = a.c[cq] + row * ny;
   float v[R];
 #pragma unroll
   for (int t = 0; t < R; ++t) {
-    const int j = q * m - d + t;
+    const int j = a.q * m - a.d + t;
     v[t] = (j >= 0 && j < ny) ? cr[j] : 0.f;
   }
-  float* o = T + gid * R;
+  float* o = a.T[cq] + gid * R;
   if constexpr (R == 4) {
     *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
   } else {
 #pragma unroll
     for (int t = 0; t < R; t += 2) *reinterpret_cast<float2*>(o + t) = make_float2(v[t], v[t + 1]);
   }
-}
-
-// The float32 V^(s) coupling on staged sources: the R y taps of a source row are one aligned vector load
-// (float4 for R = 4, three float2 for R = 6) instead of R scattered 4-byte loads.
-template <int R>
-__global__ void __launch_bounds__(128) k_apply_coupling_staged(CouplingArgs<float> a) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= a.n_act) return;
-  float acc[kMaxM];
-#pragma unroll
-  for (int m = 0; m < kMaxM; ++m) acc[m] = 0.f;
-  for (int s = 0; s < a.ns; ++s) {
-    const int bz = a.base[s][p], bx = a.base[s][a.n_act + p], by = a.base[s][2 * a.n_act + p];
-    float vz[R], vx[R], vy[R];
-    int iz[R], ix[R];
-#pragma unroll
-    for (int t = 0; t < R; ++t) {
-      vz[t] = a.val[s][(0 * R + t) * (int64_t)a.n_act + p];
-      vx[t] = a.val[s][(1 * R + t) * (int64_t)a.n_act + p];
-      vy[t] = a.val[s][(2 * R + t) * (int64_t)a.n_act + p];
-      iz[t] = min(max(bz + t, 0), a.snz[s] - 1);
-      ix[t] = min(max(bx + t, 0), a.snx[s] - 1);
-    }
-    // y interval of the point (a point outside the source box has base 0 and zero values)
-    const int my = min(max((by + a.sdir) / a.sq, 0), a.snint[s] - 1);
-    for (int jM = 0; jM < a.nM; ++jM) {
-      const float* tb = a.stage[s] + (int64_t)jM * a.snz[s] * a.snx[s] * a.snint[s] * R;
-      float sz = 0.f;
-#pragma unroll
-      for (int tz = 0; tz < R; ++tz) {
-        float sx = 0.f;
-#pragma unroll
-        for (int tx = 0; tx < R; ++tx) {
-          const float* row = tb + (((int64_t)iz[tz] * a.snx[s] + ix[tx]) * a.snint[s] + my) * R;
-          float sy;
-          if constexpr (R == 4) {
-            const float4 c4 = __ldg(reinterpret_cast<const float4*>(row));
-            sy = vy[0] * c4.x;
-            sy = fmaf(vy[1], c4.y, sy);
-            sy = fmaf(vy[2], c4.z, sy);
-            sy = fmaf(vy[3], c4.w, sy);
-          } else {
-            sy = 0.f;
-#pragma unroll
-            for (int t = 0; t < R; t += 2) {
-              const float2 c2 = __ldg(reinterpret_cast<const float2*>(row + t));
-              sy = fmaf(vy[t], c2.x, sy);
-              sy = fmaf(vy[t + 1], c2.y, sy);
-            }
-          }
-          sx = fmaf(vx[tx], sy, sx);
-        }
-        sz = fmaf(vz[tz], sx, sz);
-      }
-      for (int iM = 0; iM < a.nM; ++iM)
-        acc[iM] = fmaf(a.w[s][(int64_t)(iM * a.nM + jM) * a.n_act + p], sz, acc[iM]);
-    }
-  }
-  const int pt = a.act_pt[p];
-  for (int iM = 0; iM < a.nM; ++iM) a.y[a.row_off + (int64_t)iM * a.npts + pt] += acc[iM];
 }
 
 // ---------------------------------------------------------------------------
@@ -1853,6 +1914,87 @@ static int apply_planes(fm_ctx* c, double E, const T* x, T* y, bool only_S, T* P
   return FM_OK;
 }
 
+// y += the V^(s) coupling of x, every component in one launch (float32: on sources regrouped by y interval first).
+template <typename T>
+static int apply_coupling(fm_ctx* c, const T* x, T* y, bool timed) {
+  const int RT = c->comps[0].r;
+  if constexpr (std::is_same<T, float>::value) {
+    StageArgs st;
+    std::memset(&st, 0, sizeof(st));
+    int64_t most = 0;
+    double bytes = 0.0;
+    for (size_t k = 0; k < c->comps.size(); ++k) {
+      const Comp& cp = c->comps[k];
+      st.c[k] = x + cp.off;
+      st.T[k] = c->ystage32 + cp.ystage_off;
+      st.rows[k] = (int64_t)c->nM * cp.nz * cp.nx;
+      st.ny[k] = cp.ny;
+      st.nint[k] = cp.ay.nint;
+      most = std::max(most, st.rows[k] * cp.ay.nint);
+      bytes += 4.0 * (double)st.rows[k] * (cp.ny + (double)cp.ay.nint * RT);
+    }
+    st.q = c->comps[0].ay.q;
+    st.d = 1;
+    const dim3 g((unsigned)((most + 255) / 256), (unsigned)c->comps.size());
+    const int tk_ = timed ? prof_begin(c, FM_KERNEL_COUPLING) : -1;
+    if (RT == 6) k_stage_ytaps<6><<<g, 256, 0, c->stream>>>(st);
+    else k_stage_ytaps<4><<<g, 256, 0, c->stream>>>(st);
+    prof_end(c, tk_, 0.0, bytes);
+    c->launches++;
+  }
+  CplArgs<T> a;
+  std::memset(&a, 0, sizeof(a));
+  a.nM = c->nM;
+  a.sdir = 1;
+  a.sq = c->comps[0].ay.q;
+  int grid = 0;
+  double fl = 0.0, by = 0.0;
+  for (auto& cp : c->comps) {
+    if (cp.n_act == 0 || cp.sources.empty()) continue;
+    const ApplyTabs<T> tb = tabs_of<T>(cp);
+    CplComp<T>& f = a.c[a.ncomp++];
+    f.y = y + cp.off; f.npts = cp.npts; f.n_act = cp.n_act; f.act_pt = cp.act_pt; f.ns = (int)cp.sources.size();
+    f.mirror = cp.cpl_mirror ? 1 : 0; f.nz = cp.nz; f.nxy = cp.n_act / cp.nz; f.first = grid;
+    for (int s = 0; s < f.ns; ++s) {
+      const Comp& src = c->comps[cp.sources[s].src];
+      CplSource<T>& q = f.s[s];
+      const int tab = cp.cpl_mirror ? 0 : s;  // mirrored: source 0's taps serve both
+      q.base = cp.cpl_base + (int64_t)tab * 3 * cp.n_act;
+      q.val = tb.cval + (int64_t)tab * 3 * RT * cp.n_act;
+      q.w = tb.cw + (int64_t)s * c->nM * c->nM * cp.n_act;
+      q.src = x + src.off; q.npts = src.npts; q.nx = src.nx; q.ny = src.ny; q.nz = src.nz; q.nint = src.ay.nint;
+      if constexpr (std::is_same<T, float>::value) q.stage = c->ystage32 + src.ystage_off;
+    }
+    const int64_t items = cp.cpl_mirror ? (int64_t)(cp.nz / 2) * f.nxy : cp.n_act;
+    grid += (int)((items + 127) / 128);
+    // per evaluation 2 (R^3 + R^2 + R) flops per M'', per point and source 2 n_M^2 for the weights
+    const double cfl = 2.0 * (RT * RT * RT + RT * RT + RT) * c->nM;
+    fl += (double)cp.n_act * (cfl * (cp.cpl_mirror ? 1 : f.ns) + 2.0 * f.ns * c->nM * c->nM);
+    by += (double)cp.n_act * (4.0 + 2.0 * c->nM * sizeof(T) +
+                              (cp.cpl_mirror ? 1 : f.ns) * (12.0 + 3.0 * RT * sizeof(T)) + f.ns * c->nM * c->nM * sizeof(T));
+  }
+  if (grid == 0) return FM_OK;
+  const int tk_ = timed ? prof_begin(c, FM_KERNEL_COUPLING) : -1;
+  switch ((RT == 6 ? 8 : 0) + (c->nM <= 5 ? c->nM : 0)) {
+    case 0: k_apply_coupling<4, 0, T><<<grid, 128, 0, c->stream>>>(a); break;
+    case 1: k_apply_coupling<4, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
+    case 2: k_apply_coupling<4, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
+    case 3: k_apply_coupling<4, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
+    case 4: k_apply_coupling<4, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
+    case 5: k_apply_coupling<4, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
+    case 9: k_apply_coupling<6, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
+    case 10: k_apply_coupling<6, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
+    case 11: k_apply_coupling<6, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
+    case 12: k_apply_coupling<6, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
+    case 13: k_apply_coupling<6, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
+    default: k_apply_coupling<6, 0, T><<<grid, 128, 0, c->stream>>>(a); break;
+  }
+  prof_end(c, tk_, fl, by);
+  c->launches++;
+  FM_CUDA(cudaGetLastError());
+  return FM_OK;
+}
+
 // y = (H - E S) x (only_S: y = S x) in the element type T; scratch planes P and Q for the two-pass local form.
 template <typename T>
 static int apply_t(fm_ctx* c, double E, const T* x, T* y, bool only_S, T* P, T* Q, bool timed) {
@@ -1863,66 +2005,7 @@ static int apply_t(fm_ctx* c, double E, const T* x, T* y, bool only_S, T* P, T* 
     if (one_pass && (rc = apply_local32(c, E, x, y, only_S, timed))) return rc;
   }
   if (!one_pass && (rc = apply_planes<T>(c, E, x, y, only_S, P, Q, timed))) return rc;
-  const bool staged = std::is_same<T, float>::value && c->ystage32 != nullptr;
-  if (!only_S && staged) {  // float32: regroup every source component's y coefficients by y interval
-    for (auto& cp : c->comps) {
-      const int64_t rows = (int64_t)c->nM * cp.nz * cp.nx, items = rows * cp.ay.nint;
-      const int tk_ = timed ? prof_begin(c, FM_KERNEL_COUPLING) : -1;
-      const float* xs = reinterpret_cast<const float*>(x) + cp.off;
-      float* ts = c->ystage32 + cp.ystage_off;
-      if (cp.r == 6) k_stage_ytaps<6><<<(unsigned)((items + 255) / 256), 256, 0, c->stream>>>(xs, ts, rows, cp.ny, cp.ay.nint, cp.ay.q, 1);
-      else k_stage_ytaps<4><<<(unsigned)((items + 255) / 256), 256, 0, c->stream>>>(xs, ts, rows, cp.ny, cp.ay.nint, cp.ay.q, 1);
-      prof_end(c, tk_, 0.0, (double)rows * cp.ny * 4.0 + (double)items * cp.r * 4.0);
-      c->launches++;
-    }
-  }
-  if (!only_S) {
-    for (auto& cp : c->comps) {
-      if (cp.n_act == 0 || cp.sources.empty()) continue;
-      const ApplyTabs<T> tb = tabs_of<T>(cp);
-      CouplingArgs<T> a{};
-      a.x = x; a.y = y; a.row_off = cp.off; a.npts = cp.npts; a.n_act = cp.n_act; a.act_pt = cp.act_pt;
-      a.ns = (int)cp.sources.size(); a.nM = c->nM;
-      const int RT = cp.r;
-      for (int s = 0; s < a.ns; ++s) {
-        const auto& src = c->comps[cp.sources[s].src];
-        a.base[s] = cp.cpl_base + (int64_t)s * 3 * cp.n_act;
-        a.val[s] = tb.cval + (int64_t)s * 3 * RT * cp.n_act;
-        a.w[s] = tb.cw + (int64_t)s * c->nM * c->nM * cp.n_act;
-        a.src_off[s] = src.off; a.src_npts[s] = src.npts;
-        a.snx[s] = src.nx; a.sny[s] = src.ny; a.snz[s] = src.nz;
-        if (staged) {
-          a.stage[s] = reinterpret_cast<const T*>(c->ystage32 + src.ystage_off);
-          a.snint[s] = src.ay.nint;
-        }
-      }
-      a.sdir = 1;
-      a.sq = cp.ay.q;
-      {
-        const int tk_ = timed ? prof_begin(c, FM_KERNEL_COUPLING) : -1;
-        if constexpr (std::is_same<T, float>::value) {
-          if (staged) {
-            if (RT == 6) k_apply_coupling_staged<6><<<(cp.n_act + 127) / 128, 128, 0, c->stream>>>(a);
-            else k_apply_coupling_staged<4><<<(cp.n_act + 127) / 128, 128, 0, c->stream>>>(a);
-          } else if (RT == 6) {
-            k_apply_coupling<6, T><<<(cp.n_act + 127) / 128, 128, 0, c->stream>>>(a);
-          } else {
-            k_apply_coupling<4, T><<<(cp.n_act + 127) / 128, 128, 0, c->stream>>>(a);
-          }
-        } else {
-          if (RT == 6) k_apply_coupling<6, T><<<(cp.n_act + 127) / 128, 128, 0, c->stream>>>(a);
-          else k_apply_coupling<4, T><<<(cp.n_act + 127) / 128, 128, 0, c->stream>>>(a);
-        }
-        // per (point, source): 2 (R^3 + R^2 + R) contraction flops per M'' and 2 n_M^2 for the weights
-        const double cfl = 2.0 * (RT * RT * RT + RT * RT + RT);
-        prof_end(c, tk_, (double)cp.n_act * a.ns * (cfl * c->nM + 2.0 * c->nM * c->nM),
-                 (double)cp.n_act * (4.0 + 2.0 * c->nM * sizeof(T) + a.ns * (12.0 + (3.0 * RT + c->nM * c->nM) * sizeof(T))));
-      }
-      c->launches++;
-    }
-  }
-  FM_CUDA(cudaGetLastError());
-  return FM_OK;
+  return only_S ? FM_OK : apply_coupling<T>(c, x, y, timed);
 }
 
 int launch_apply(fm_ctx* c, double E, const double* x, double* y, bool only_S) {

@@ -424,6 +424,21 @@ static bool tc_requested(const fm_ctx* c) {
   return c->opts.precision != FM_PREC_FP64 && c->opts.mma != FM_MMA_SIMT;
 }
 
+// Whether sources 0 and 1 of a component can share their taps: the expansion of one component at +z and, by the
+// exchange symmetry, at -z, rotations that differ in the sign of s, z points symmetric to rounding.
+static bool cp_mirror(const fm_ctx* c, const Comp& cp) {
+  if (cp.sources.size() != 2 || cp.nz % 2 != 0) return false;
+  const Source &a = cp.sources[0], &b = cp.sources[1];
+  if (a.src != b.src || a.zsign != 1.0 || b.zsign != -1.0) return false;
+  double ca, sa, cb, sb;
+  rotation(c->sys.mass, a.beta, cp.label, &ca, &sa);
+  rotation(c->sys.mass, b.beta, cp.label, &cb, &sb);
+  if (ca != cb || sa != -sb) return false;
+  for (int k = 0; k < cp.nz; ++k)
+    if (std::fabs(cp.az.pts[k] + cp.az.pts[cp.nz - 1 - k]) > 1e-15) return false;
+  return true;
+}
+
 int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
   const fm_system& S = c->sys;
   const double* m = S.mass;
@@ -631,9 +646,13 @@ int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
             if (on_xy[(size_t)i * cp.ny + j]) act.push_back((int)(((int64_t)k * cp.nx + i) * cp.ny + j));
       cp.n_act = (int)act.size();
       const int ns = (int)cp.sources.size(), na = cp.n_act;
-      std::vector<int> base((size_t)ns * 3 * na);
+      // sources 0 and 1 the same expansion seen from the two particles of the identical pair, on a z grid
+      // symmetric about 0: source 1 at (x, y, z) is source 0 at (x, y, -z)
+      cp.cpl_mirror = cp_mirror(c, cp);
+      const int nt = cp.cpl_mirror ? 1 : ns;  // sets of taps
+      std::vector<int> base((size_t)nt * 3 * na);
       const int R = cp.r, R3 = 3 * cp.r;
-      std::vector<double> val((size_t)ns * R3 * na), wt((size_t)ns * nM * nM * na);
+      std::vector<double> val((size_t)nt * R3 * na), wt((size_t)ns * nM * nM * na);
       std::atomic<int> bad_w{0};
       const int chunk = 4096, nchunks = (na + chunk - 1) / chunk;
       for (int s = 0; s < ns; ++s) {
@@ -649,13 +668,16 @@ int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
           double xb, yb, zb;
           rotate(cc, ss, x, y, z, &xb, &yb, &zb);
           const double w = w_angle(src.beta, cp.label, cc, ss, x, y, z, yb);
-          int b3[3];
-          double v[3 * kMaxTaps];
-          sc.az.eval(src.zsign * zb, 0, &b3[0], v);
-          sc.ax.eval(xb, 0, &b3[1], v + R);
-          sc.ay.eval(yb, 0, &b3[2], v + 2 * R);
-          for (int d = 0; d < 3; ++d) base[((size_t)s * 3 + d) * na + p] = b3[d];
-          for (int t = 0; t < R3; ++t) val[((size_t)s * R3 + t) * na + p] = v[t];
+          if (s < nt) {
+            int b3[3];
+            double v[3 * kMaxTaps];
+            sc.az.eval(src.zsign * zb, 0, &b3[0], v);
+            sc.ax.eval(xb, 0, &b3[1], v + R);
+            sc.ay.eval(yb, 0, &b3[2], v + 2 * R);
+            if (!(xb >= sc.ax.a && xb <= sc.ax.b && yb >= sc.ay.a && yb <= sc.ay.b)) b3[0] = -1;  // zero there
+            for (int d = 0; d < 3; ++d) base[((size_t)s * 3 + d) * na + p] = b3[d];
+            for (int t = 0; t < R3; ++t) val[((size_t)s * R3 + t) * na + p] = v[t];
+          }
           // weight V^(s)_a * rho * rho^{M''} * angular(M', M'') * [p (-1)^{M''}]
           const double vc = coulomb(c, cp.label, x);
           const double vs = (c->split.mode == FM_SPLIT_MERKURIEV) ? chi(c->split, x, y) * vc : vc;
