@@ -624,6 +624,8 @@ int fm_create(const fm_system* sys, const fm_grid* grids, int n_grids, const fm_
       (rc = dev_alloc(c, (void**)&c->gs_cnt, 256)) || (rc = dev_alloc(c, (void**)&c->tuneG_dev, 64 * 8)))
     return fail(rc);
   if (cudaMemset(c->gs_cnt, 0, 256) != cudaSuccess) return fail(FM_ERR_CUDA);
+  c->tc_err = tc_flag_slot(c);  // flag of an expired wait, read back with every Gram-Schmidt result
+  if (cudaMemsetAsync(c->tc_err, 0, 2 * sizeof(int), c->stream) != cudaSuccess) return fail(FM_ERR_CUDA);
   if (cudaMallocHost((void**)&c->red_host, 8192 * 8) != cudaSuccess) return fail(FM_ERR_OOM);
   if (c->use_dd) {  // double-float Krylov workspace; float32 buffers of the preconditioner's input and output
     if ((rc = dev_alloc(c, (void**)&c->Vdd, (size_t)(m + 1) * N * 8)) || (rc = dev_alloc(c, (void**)&c->Zdd, (size_t)m * N * 8)) ||

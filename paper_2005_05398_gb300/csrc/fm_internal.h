@@ -36,10 +36,13 @@ struct Axis {
 
 // Half-width of the banded y systems of one l (Section 3.2, the M' chain of n_c components interleaved
 // with y): the 1D band of the y collocation matrices times n_c, plus the M' coupling to the neighbours.
-inline int band_kl(const Axis& ay, int nc) {
+// At least 2 (cubic) or 4 (quintic) even on a single interval, so that the y-solve kernel's band widths are the
+// same set for every grid.
+inline int band_kq(const Axis& ay) {
   const int k = ay.kl > ay.ku ? ay.kl : ay.ku;
-  return nc == 1 ? k : k * nc + 1;
+  return k > (ay.q == 2 ? 2 : 4) ? k : (ay.q == 2 ? 2 : 4);
 }
+inline int band_kl(const Axis& ay, int nc) { return nc == 1 ? band_kq(ay) : band_kq(ay) * nc + 1; }
 constexpr int kMaxBandKL = 25;  // widest banded y system the y-solve kernel takes
 
 // Device-side 1D tap tables of one axis.
@@ -116,12 +119,13 @@ struct Comp {
   // preconditioner, E-dependent banded y systems: per l a group of nx lines
   std::vector<int> chain_lo, chain_n;   // per l: first iM and length of the M' chain
   int* d_chain_lo = nullptr; int* d_chain_n = nullptr;
-  int64_t* d_band_off = nullptr; int64_t* d_lmul_off = nullptr; int64_t* d_piv_off = nullptr;
+  int* d_pstep = nullptr;               // per l: n_c when every pivot offset is a multiple of it, else 1
+  int64_t* d_band_off = nullptr; int64_t* d_lmul_off = nullptr;
   std::vector<int64_t> band_off;        // per l: offset (in elements) of its group in yU / yL
-  std::vector<int64_t> piv_off;
-  int64_t band_total = 0, lmul_total = 0, piv_total = 0;
-  double* yU = nullptr;          // per l: [n][kl+ku+1][nx], reciprocal pivot first
-  double* yL = nullptr;          // per l: [n][kl+1][nx], slot 0 the pivot offset, then the multipliers
+  int64_t band_total = 0, lmul_total = 0;
+  // per l and block of 32 lines (the last one padded to a multiple of 4), in the order of the sweeps:
+  double* yU = nullptr;          // [n, last row first][kl+ku+1][lines]: reciprocal pivot, then U[r - d][r]
+  double* yL = nullptr;          // [n][kl+1][lines]: pivot offset (an integer's bits), then the multipliers
   float* yU32 = nullptr; float* yL32 = nullptr;
   std::vector<int64_t> lmul_off;
   // n_M = 1: per-l diagonalisation of (A_l, S_y), A_l = -D_y + (c_l Y_r2 + V^ - E*) S_y, used by the

@@ -828,8 +828,8 @@ int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
     cp.chain_n.assign(nl, 0);
     cp.band_off.assign(nl, 0);
     cp.lmul_off.assign(nl, 0);
-    cp.piv_off.assign(nl, 0);
-    int64_t bo = 0, lo = 0, po = 0;
+    int64_t bo = 0, lo = 0;
+    const int nxp = (nx + 3) / 4 * 4;  // lines as stored
     for (int il = 0; il < nl; ++il) {
       const int l = c->M0 + il;
       int first = -1, cnt = 0;
@@ -846,19 +846,16 @@ int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
       if (kl > kMaxBandKL) return FM_ERR_ARG;  // M' chain too long for the banded y solve of this basis
       cp.band_off[il] = bo;
       cp.lmul_off[il] = lo;
-      cp.piv_off[il] = po;
-      bo += (int64_t)n * (2 * kl + 1) * nx;
-      lo += (int64_t)n * (kl + 1) * nx;
-      po += (int64_t)n * nx;
+      bo += (int64_t)n * (2 * kl + 1) * nxp;
+      lo += (int64_t)n * (kl + 1) * nxp;
     }
     cp.band_total = bo;
     cp.lmul_total = lo;
-    cp.piv_total = po;
     if ((rc = upload(c, (void**)&cp.d_chain_lo, cp.chain_lo.data(), nl * sizeof(int)))) return rc;
     if ((rc = upload(c, (void**)&cp.d_chain_n, cp.chain_n.data(), nl * sizeof(int)))) return rc;
     if ((rc = upload(c, (void**)&cp.d_band_off, cp.band_off.data(), nl * sizeof(int64_t)))) return rc;
     if ((rc = upload(c, (void**)&cp.d_lmul_off, cp.lmul_off.data(), nl * sizeof(int64_t)))) return rc;
-    if ((rc = upload(c, (void**)&cp.d_piv_off, cp.piv_off.data(), nl * sizeof(int64_t)))) return rc;
+    if ((rc = dev_alloc(c, (void**)&cp.d_pstep, nl * sizeof(int)))) return rc;
     if ((rc = dev_alloc(c, (void**)&cp.yU, bo * 8))) return rc;
     if ((rc = dev_alloc(c, (void**)&cp.yL, lo * 8))) return rc;
     if ((rc = dev_alloc(c, (void**)&cp.yU32, bo * 4))) return rc;
@@ -936,8 +933,8 @@ int estimate_bytes(const fm_system* S, const fm_grid* grids, int n_grids, const 
         if (Mp <= l && l <= Mp + (int)nz - 1) ++cnt;
       }
       const double n = cnt * ny, kl = band_kl(ay, cnt);
-      bo += n * (2 * kl + 1) * nx;
-      lo += n * (kl + 1) * nx;
+      bo += n * (2 * kl + 1) * ((ax.n + 3) / 4 * 4);
+      lo += n * (kl + 1) * ((ax.n + 3) / 4 * 4);
     }
     bytes += bo * 12.0 + lo * 12.0;
     if (nM == 1) bytes += 2.0 * nl * ny * ny * 12.0 + nl * (nx + ny) * 20.0;  // per-l y diagonalisation
@@ -963,7 +960,7 @@ int estimate_bytes(const fm_system* S, const fm_grid* grids, int n_grids, const 
 // system with banded blocks N^{M'}_{l i} = A1 + (J(J+1) - 2M'^2 + l(l+1)) A2 and
 // N^{M'+-} = (off-diagonal coefficient) A2, where A1 = -D_y + V^ S_y - E* S_y +
 // (Lambda_x^l)_{ii} S_y and A2 = Y_r2 S_y (Section 3.2, Eq. ops and the matrix L0).
-// Factorised by banded LU with the unknowns ordered r = j * n_c + c.
+// Factorised by banded LU with the unknowns ordered r = j * n_c + c, stored in the order the sweeps read them.
 int setup_shift(fm_ctx* c, double Estar) {
   const int J = c->sys.J;
   int rc;
@@ -971,6 +968,8 @@ int setup_shift(fm_ctx* c, double Estar) {
   for (auto& cp : c->comps) {
     const int nx = cp.nx, ny = cp.ny;
     std::vector<double> U((size_t)cp.band_total), L((size_t)cp.lmul_total);
+    std::vector<float> U32(U.size()), L32(L.size());
+    std::vector<int> pstep(cp.nl);
     std::vector<double> vh(ny);
     for (int j = 0; j < ny; ++j) vh[j] = vhat(c, cp.label, cp.ay.pts[j], cp.Ry);
     std::vector<int> bad(cp.nl, 0);
@@ -983,6 +982,7 @@ int setup_shift(fm_ctx* c, double Estar) {
       const int R = cpp->ay.r;
       std::vector<double> B((size_t)n * wb), Lm((size_t)n * kl);
       std::vector<int> piv(n);
+      int step = nc;
       for (int ix = 0; ix < nx; ++ix) {
         const double lx = cpp->Lx[(size_t)il * nx + ix];
         std::fill(B.begin(), B.end(), 0.0);
@@ -1008,24 +1008,41 @@ int setup_shift(fm_ctx* c, double Estar) {
           bad[il] = 1;
           return;
         }
-        // per row r: U[r][0] = 1 / pivot, U[r][1..wu) the upper band; L[r][0] = pivot offset,
-        // L[r][1..kl] = multipliers
-        double* Ug = &U[cpp->band_off[il]];
-        double* Lg = &L[cpp->lmul_off[il]];
+        // the block of 32 lines this one belongs to: [row][slot][lines of the block, padded to 4]
+        const int wd = std::min(32, (nx - (ix & ~31) + 3) / 4 * 4), ln = ix & 31;
+        const size_t ub = (size_t)cpp->band_off[il] + (size_t)(ix & ~31) * n * wu + ln;
+        const size_t lb = (size_t)cpp->lmul_off[il] + (size_t)(ix & ~31) * n * (kl + 1) + ln;
         for (int r = 0; r < n; ++r) {
-          Ug[((size_t)r * wu) * nx + ix] = 1.0 / B[(size_t)r * wb + kl];  // reciprocal of the pivot
-          for (int d = 1; d < wu; ++d) Ug[((size_t)r * wu + d) * nx + ix] = B[(size_t)r * wb + kl + d];
-          Lg[((size_t)r * (kl + 1)) * nx + ix] = (double)(piv[r] - r);
-          for (int d = 0; d < kl; ++d) Lg[((size_t)r * (kl + 1) + d + 1) * nx + ix] = Lm[(size_t)r * kl + d];
+          // backward sweep, last row first: 1 / pivot of row r, then its column above, U[r - d][r]
+          const size_t u0 = ub + (size_t)(n - 1 - r) * wu * wd;
+          for (int d = 0; d < wu; ++d) {
+            const double v = d == 0 ? 1.0 / B[(size_t)r * wb + kl] : (r >= d ? B[(size_t)(r - d) * wb + kl + d] : 0.0);
+            U[u0 + (size_t)d * wd] = v;
+            U32[u0 + (size_t)d * wd] = (float)v;
+          }
+          // forward sweep: the pivot offset as integer bits, then the multipliers
+          const size_t l0 = lb + (size_t)r * (kl + 1) * wd;
+          const int32_t pv = piv[r] - r;
+          const int64_t pv64 = pv;
+          std::memcpy(&L[l0], &pv64, 8);
+          std::memcpy(&L32[l0], &pv, 4);
+          if (pv % nc != 0) step = 1;
+          for (int d = 0; d < kl; ++d) {
+            L[l0 + (size_t)(d + 1) * wd] = Lm[(size_t)r * kl + d];
+            L32[l0 + (size_t)(d + 1) * wd] = (float)Lm[(size_t)r * kl + d];
+          }
         }
       }
+      // the kernel's instantiations with a pivot step: n_c = 2 .. 5 (cubic), 2 .. 4 (quintic)
+      const int kq = band_kq(cpp->ay);
+      pstep[il] = (nc >= 2 && nc <= (kq == 2 ? 5 : 4) && (kq == 2 || kq == 4)) ? step : 1;
     });
     for (int b : bad)
       if (b) return FM_ERR_NUMERIC;
     tm.mark("banded y factors");
     FM_CUDA(cudaMemcpyAsync(cp.yU, U.data(), U.size() * 8, cudaMemcpyHostToDevice, c->stream));
     FM_CUDA(cudaMemcpyAsync(cp.yL, L.data(), L.size() * 8, cudaMemcpyHostToDevice, c->stream));
-    std::vector<float> U32(U.begin(), U.end()), L32(L.begin(), L.end());
+    FM_CUDA(cudaMemcpyAsync(cp.d_pstep, pstep.data(), pstep.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
     FM_CUDA(cudaMemcpyAsync(cp.yU32, U32.data(), U32.size() * 4, cudaMemcpyHostToDevice, c->stream));
     FM_CUDA(cudaMemcpyAsync(cp.yL32, L32.data(), L32.size() * 4, cudaMemcpyHostToDevice, c->stream));
     FM_CUDA(cudaStreamSynchronize(c->stream));

@@ -960,10 +960,6 @@ int tc_setup(fm_ctx* c) {
   for (auto& cp : c->comps) all = all && (want_bf16 ? bf16_component_ok(cp) : tc_component_ok(cp));
   if (!all) return (c->opts.mma == FM_MMA_TF32 || want_bf16) ? FM_ERR_ARG : FM_OK;
   if (!encode_fn()) return c->opts.mma == FM_MMA_AUTO ? FM_OK : FM_ERR_CUDA;
-  if (!c->tc_err) {  // read back with every Gram-Schmidt result, so a Krylov step sees an expired wait
-    c->tc_err = tc_flag_slot(c);
-    FM_CUDA(cudaMemsetAsync(c->tc_err, 0, sizeof(double), c->stream));
-  }
   const CUtensorMapDataType dt = want_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
   const int es = want_bf16 ? 2 : 4, E = 128 / es;
   for (auto& cp : c->comps) {

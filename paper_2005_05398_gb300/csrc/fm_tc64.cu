@@ -620,8 +620,6 @@ int f64_setup(fm_ctx* c) {
   FM_CUDA(cudaFuncSetAttribute(k_tc_f64<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   FM_CUDA(cudaFuncSetAttribute(k_tc_f64<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
   FM_CUDA(cudaFuncSetAttribute(k_tc_f64<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
-  c->tc_err = tc_flag_slot(c);
-  FM_CUDA(cudaMemsetAsync(c->tc_err, 0, 2 * sizeof(int), c->stream));
   int* bad = c->tc_err + 1;
   bool all = true;
   for (auto& cp : c->comps) all = all && cp.nx <= kF64MaxK && cp.nz <= kF64MaxK;
