@@ -287,7 +287,7 @@ int fm_stats(const fm_ctx* ctx, int64_t* launches, int64_t* device_bytes);
  * and code on a time-critical path, where cudaMalloc / cudaFree can synchronise the device.
  * The paper has no counterpart: it is an interface for such callers.  The context is built
  * by fm_create beforehand (which does allocate); this call allocates nothing.  Its scratch
- * (three planes of n_unknowns doubles) is a fixed array inside the library, 24 MiB that every
+ * (two planes of n_unknowns doubles) is a fixed array inside the library, 16 MiB that every
  * GPU loading the library holds until the process exits; n_unknowns above
  * FM_NOALLOC_MAX_UNKNOWNS gives FM_ERR_SCRATCH_LIMIT.  The first call on a device looks up
  * the array's device address (cudaGetSymbolAddress, with that device current); make that first

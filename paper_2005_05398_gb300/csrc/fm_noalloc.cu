@@ -1,9 +1,9 @@
-// fm_apply_noalloc: the operator apply y = (H - E S) x with its three scratch planes taken from
+// fm_apply_noalloc: the operator apply y = (H - E S) x with its two scratch planes taken from
 // a fixed device array of this file instead of the context's own buffers.  The call performs no
 // device allocation of any kind (no cudaMalloc / cudaFree, no allocating library routine).
 //
 // The array below is part of the library image: every GPU on which the library is loaded holds
-// FM_NOALLOC_MAX_UNKNOWNS * 3 doubles (24 MiB) for it until the process exits.  Host code may not
+// FM_NOALLOC_MAX_UNKNOWNS * 2 doubles (16 MiB) for it until the process exits.  Host code may not
 // use the array's name as a device address (in host code it names a host-side stand-in), so the
 // device address is obtained once per device with cudaGetSymbolAddress, with that device current.
 #include <cuda.h>
@@ -16,7 +16,7 @@
 
 namespace {
 
-static __device__ __align__(256) double g_apply_scratch[3 * (size_t)FM_NOALLOC_MAX_UNKNOWNS];
+static __device__ __align__(256) double g_apply_scratch[2 * (size_t)FM_NOALLOC_MAX_UNKNOWNS];
 
 constexpr int kMaxDevices = 64;
 struct ScratchSlot {
