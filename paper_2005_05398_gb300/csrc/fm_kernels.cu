@@ -406,6 +406,9 @@ struct CplArgs {
 // the source's expansion of every M'' at point p; false outside its box
 template <int R, int NMC, typename T>
 __device__ __forceinline__ bool cpl_eval(const CplSource<T>& s, int p, int n_act, int nM, int sdir, int sq, T* E) {
+  // the M'' loop is rolled up for a count known only at run time: twelve bodies of r^3 taps gain
+  // nothing beside one (E[jM] is one store per body) and take the compiler minutes
+  constexpr int kUnM = NMC ? NMC : 1;
   const int bz = s.base[p];
   if (bz < 0) return false;
   const int bx = s.base[n_act + p], by = s.base[2 * n_act + p];
@@ -421,7 +424,7 @@ __device__ __forceinline__ bool cpl_eval(const CplSource<T>& s, int p, int n_act
   if constexpr (std::is_same<T, float>::value) {
     // regrouped by y interval: a source row's R taps are one aligned vector load
     const int my = min(max((by + sdir) / sq, 0), s.nint - 1);
-#pragma unroll
+#pragma unroll kUnM
     for (int jM = 0; jM < (NMC ? NMC : kMaxM); ++jM) {
       if (!NMC && jM >= nM) break;
       const float* tb = s.stage + (int64_t)jM * s.nz * s.nx * s.nint * R;
@@ -454,7 +457,7 @@ __device__ __forceinline__ bool cpl_eval(const CplSource<T>& s, int p, int n_act
     int iy[R];
 #pragma unroll
     for (int t = 0; t < R; ++t) iy[t] = min(max(by + t, 0), s.ny - 1);
-#pragma unroll
+#pragma unroll kUnM
     for (int jM = 0; jM < (NMC ? NMC : kMaxM); ++jM) {
       if (!NMC && jM >= nM) break;
       const T* cb = s.src + (int64_t)jM * s.npts;
@@ -2000,19 +2003,24 @@ static int apply_coupling(fm_ctx* c, const T* x, T* y, bool timed) {
   }
   if (grid == 0) return FM_OK;
   const int tk_ = timed ? prof_begin(c, FM_KERNEL_COUPLING) : -1;
-  switch ((RT == 6 ? 8 : 0) + (c->nM <= 5 ? c->nM : 0)) {
-    case 0: k_apply_coupling<4, 0, T><<<grid, 128, 0, c->stream>>>(a); break;
-    case 1: k_apply_coupling<4, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
-    case 2: k_apply_coupling<4, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
-    case 3: k_apply_coupling<4, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
-    case 4: k_apply_coupling<4, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
-    case 5: k_apply_coupling<4, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
-    case 9: k_apply_coupling<6, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
-    case 10: k_apply_coupling<6, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
-    case 11: k_apply_coupling<6, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
-    case 12: k_apply_coupling<6, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
-    case 13: k_apply_coupling<6, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
-    default: k_apply_coupling<6, 0, T><<<grid, 128, 0, c->stream>>>(a); break;
+  if constexpr (std::is_same<T, dd>::value) {  // any n_M: an instantiation of this type takes the compiler seconds
+    if (RT == 6) k_apply_coupling<6, 0, T><<<grid, 128, 0, c->stream>>>(a);
+    else k_apply_coupling<4, 0, T><<<grid, 128, 0, c->stream>>>(a);
+  } else {
+    switch ((RT == 6 ? 8 : 0) + (c->nM <= 5 ? c->nM : 0)) {
+      case 0: k_apply_coupling<4, 0, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 1: k_apply_coupling<4, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 2: k_apply_coupling<4, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 3: k_apply_coupling<4, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 4: k_apply_coupling<4, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 5: k_apply_coupling<4, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 9: k_apply_coupling<6, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 10: k_apply_coupling<6, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 11: k_apply_coupling<6, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 12: k_apply_coupling<6, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 13: k_apply_coupling<6, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
+      default: k_apply_coupling<6, 0, T><<<grid, 128, 0, c->stream>>>(a); break;
+    }
   }
   prof_end(c, tk_, fl, by);
   c->launches++;
