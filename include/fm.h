@@ -107,7 +107,9 @@ enum { FM_PREC_FP64 = 0, FM_PREC_FP32 = 1, FM_PREC_MIXED = 2 };
  * and, with n_M = 1, the fused x / y chain; the x stages around the banded y solves (n_M > 1) stay
  * TF32; needs n_x, n_y multiples of 8 in [16, 256] and n_z <= 128 (else FM_ERR_ARG).
  * Float64 preconditioner (FP64 precision): its z and x mode products run on the tensor cores as exact products
- * of integer digits (at least float64 accuracy) where n_x and n_z are at most 256; with SIMT on the CUDA cores.
+ * of integer digits where n_x and n_z are at most 256 (in the 2-norm of each M' component no less accurate than
+ * float64 multiply-adds; an entry far below the largest of its line has that line's last bits); with SIMT on
+ * the CUDA cores.
  * On the tensor cores the z stages run as tcgen05 GEMMs when n_z <= 128, and for n_M = 1 the x and y
  * stages of one slab (z mode) run in one kernel that keeps the slab on chip. */
 enum { FM_MMA_AUTO = 0, FM_MMA_SIMT = 1, FM_MMA_TF32 = 2, FM_MMA_BF16 = 3 };

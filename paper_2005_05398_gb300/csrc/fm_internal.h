@@ -77,6 +77,7 @@ struct TabsDD {
 struct F64Mat {
   CUtensorMap tm;                // digits [nl * 7][n][n padded to 8], float16
   int* exps = nullptr;           // [nl][n] row exponents
+  int* bal = nullptr;            // z inverse: [nl][n] exponents its columns were lowered by (<< 20)
   const double* W = nullptr;     // the matrices
 };
 

@@ -939,7 +939,7 @@ int estimate_bytes(const fm_system* S, const fm_grid* grids, int n_grids, const 
     bytes += bo * 12.0 + lo * 12.0;
     if (nM == 1) bytes += 2.0 * nl * ny * ny * 12.0 + nl * (nx + ny) * 20.0;  // per-l y diagonalisation
     if (o->precision == FM_PREC_FP64 && o->mma != FM_MMA_SIMT)                                 // digits of the tensor-core stages
-      bytes += 2.0 * (f64_digit_bytes(nM, az.n) + f64_digit_bytes((int64_t)nl, ax.n));
+      bytes += 2.0 * (f64_digit_bytes(nM, az.n) + f64_digit_bytes((int64_t)nl, ax.n)) + 4.0 * nM * az.n;
     if (o->precision != FM_PREC_FP64 && o->mma != FM_MMA_SIMT) {
       bytes += 2.0 * nM * nz * (nz + 8) * 4.0;                           // padded z factors of the tensor cores
       if (o->mma == FM_MMA_BF16) bytes += 2.0 * nl * (nx * nx + (nM == 1 ? ny * ny : 0.0)) * 2.0;

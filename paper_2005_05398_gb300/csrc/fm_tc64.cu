@@ -4,19 +4,26 @@
 // the float64 CUDA-core kernels (k_zmix, k_mix) spend 0.70 + 2.4 ms on them per application at 3.7 M unknowns
 // (He L=0, 96 x 96 x 24 intervals).  Here both operands are split into integer digits whose products the tensor
 // cores add exactly (Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012; Mukunoki et al., ISC 2020):
-//   * a row of W and a column of the slab are scaled by a power of two (its largest entry) to 56-bit integers,
-//     seven balanced base-256 digits d_0 .. d_6 in [-128, 128], each exact in float16;
+//   * a row of W and a column of the slab are scaled by a power of two (its largest entry) to integers of 62 bits
+//     (K <= 64) or 59 bits, seven balanced base-512 digits d_0 .. d_6 in [-256, 256], each exact in float16;
 //   * the 34 products with i + j <= 7 run as tcgen05.mma kind::f16, those of one weight g = i + j into one
-//     float32 accumulator D_g (8 accumulators in tensor memory).  |D_g| <= (g + 1) K 2^14 <= 2^24 for g <= 3 at
-//     K <= 256, so these are exact; a rounding of D_4 .. D_7 beyond 2^24 is at most 2^-46 of the row's and
-//     column's maxima, below the K 2^-53 of a float64 sum of that size;
-//   * the epilogue adds sum_g 2^(8 (6 - g)) D_g as a fixed-point integer and rounds once to float64, in integer
+//     float32 accumulator D_g (8 accumulators in tensor memory).  A float32 sum of integers is exact up to 2^24:
+//     |D_g| <= (g + 1) K 2^16 for K <= 64, so D_0 .. D_3 are; above, |d_0| <= 32 keeps D_0 and D_1 exact for any
+//     input, and the split of W checks D_2 and D_3 from the digit sums of its rows (K > 192: each half of K has
+//     accumulators of its own).  Beyond 2^24 a rounding of D_4 .. D_7 costs 2^-43 of the row's and column's maxima or
+//     less; it takes slab digits that follow the signs of hundreds of digits of W (sums are about 2^19 otherwise);
+//   * the epilogue adds sum_g 2^(9 (7 - g)) D_g as a fixed-point integer and rounds once to float64, in integer
 //     arithmetic (the FP64 pipe is not touched).
-// Against 80-bit sums of the solver's own matrices (He and Ps- grids, both bases, z and x stages, N(0,1) vectors
-// through the chain) the relative 2-norm error is 5e-17 .. 1e-16, that of the float64 fused multiply-add chain
-// 1.0e-16 .. 4.7e-16; with the weights g <= 6 alone it was 1e-16 .. 5e-16.  A column with an infinity, a NaN or
-// a maximum outside 2^+-677 takes a float64 loop over the original values instead, so every input the CUDA-core
-// kernels took gives what it gave.
+// The columns of W_z are scaled to g_l^{M'}(1) and span up to 1e8 while the modes they meet are damped at high l: on
+// the scale of the column's largest mode the products that matter would be cut off (base 256 without balance lost
+// 1e-14 .. 6e-10 there).  The z inverse therefore takes column k of W_z by 2^-a_k and mode k of the slab by 2^a_k, a_k
+// the exponent of that column's maximum: an integer add per value.
+// Accuracy, against 64-bit-mantissa sums of the solver's own matrices, over both bases, J <= 10, n_z = 8 .. 130,
+// n_x = 48 .. 256, with random and with smooth vectors taken through the chain (relative 2-norm per M' component):
+// z stages 3e-17 .. 1e-16 where the float64 chain has 6e-17 .. 1.7e-15 (K > 64: up to 1.6e-15 against 2.3e-15), x
+// stages 5e-17 .. 1.3e-15 against 1e-16 .. 1.6e-15.  The bound is normwise: an entry far below its column's largest
+// product carries that product's last bits.  A column with an infinity, a NaN or a maximum outside 2^+-677 takes a
+// float64 loop over the original values instead.
 //
 // One CTA per SM walks (slab, column tile) pairs: 16 worker warps load the tile's doubles (the next tile's are in
 // flight during the MMAs), split them into K-major 128-byte-swizzled operands that stay for every row tile, and
@@ -46,7 +53,7 @@ namespace fmi {
 
 namespace {
 
-constexpr int kDig = 7;             // base-256 digits per value
+constexpr int kDig = 7;             // base-512 digits per value
 constexpr int kAcc = 8;             // accumulators: weights g = i + j = 0 .. 7
 constexpr int kWorkers = 512;       // load / split / epilogue threads
 constexpr int kProducer = kWorkers / 32, kIssuer = kProducer + 1;  // warps
@@ -57,6 +64,7 @@ struct F64Comp {
   CUtensorMap tmA;         // digits of W: [nl * 7][rows][ld], box 64 x 128
   const double* W;         // [nl][M][M]
   const int* expA;         // [nl][M] biased exponent of the row maximum
+  const int* bal;          // z inverse: [nl][M] exponents a_k the slab's values are raised by (<< 20), else null
   const double* in;
   double* out;
   int K, N;                // contraction length (= rows of W), columns
@@ -94,66 +102,69 @@ __device__ __forceinline__ bool named_sync_or(int id, int nthreads, bool v) {
   return r != 0;
 }
 
-// The 56-bit integer of a double on the scale of a maximum with biased exponent 'emax' (2^(54 + 1023 - emax)
-// times the value, rounded to nearest), plus 0x80 in every digit: byte 6 - i (and bit 56) of the result, less
-// 128, is digit d_i.
-__device__ __forceinline__ uint64_t digits_of(double v, int emax) {
+// bits of a value of 1 on the integers' scale: 62-bit integers for K <= 64, 59-bit ones (|d_0| <= 32) otherwise
+constexpr int kBitsSmall = 61, kBitsLarge = 58;
+
+// The integer of a double on the scale of a maximum with biased exponent 'emax' (2^(bits + 1023 - emax) times the
+// value, rounded to nearest), plus 256 in every digit: bits 9 (6 - i) .. + 8 of the result (d_0: ten bits), less
+// 256, are digit d_i.
+__device__ __forceinline__ uint64_t digits_of(double v, int emax, int bits) {
   const uint64_t b = (uint64_t)__double_as_longlong(v);
   const int e = (int)((b >> 52) & 0x7FF);
   uint64_t m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-  const int sh = emax - 2 - e;
+  const int sh = emax - (bits - 52) - e;
   if (e == 0 || sh > 54) m = 0;  // zero, denormal or below half a unit
   else if (sh <= 0) m <<= -sh;
   else m = (m + (1ull << (sh - 1))) >> sh;
   if ((int64_t)b < 0) m = 0ull - m;
-  return m + 0x80808080808080ull;
+  return m + 0x4020100804020100ull;
 }
 
-// The same for the slab's values, truncated toward zero, in 32-bit words with few ALU instructions (that pipe
-// bounds the splitting: the 64-bit form above took 83 of them a value, this one 15).  The error is below one
-// unit, 2^-55 of the column's maximum.  emax of an all-zero column must be large.
-__device__ __forceinline__ void digits32(double v, uint32_t emax, uint32_t& lo, uint32_t& hi) {
-  const uint32_t bh = (uint32_t)__double2hiint(v), bl = (uint32_t)__double2loint(v);
-  const uint32_t mh = __funnelshift_l(bl, (bh & 0xFFFFFu) | 0x100000u, 2), ml = bl << 2;
+// The same for the slab's values (high and low word), truncated toward zero, in 32-bit words with few ALU
+// instructions (that pipe bounds the splitting).  The error is below one unit, 2^-bits of the column's maximum.
+// emax of an all-zero column must be large.
+template <int BITS>
+__device__ __forceinline__ void digits32(uint32_t bh, uint32_t bl, uint32_t emax, uint32_t& lo, uint32_t& hi) {
+  const uint32_t mh = __funnelshift_l(bl, (bh & 0xFFFFFu) | 0x100000u, BITS - 52), ml = bl << (BITS - 52);
   const uint32_t sh = emax - ((bh >> 20) & 0x7FFu);  // >= 0; an exponent of 0 shifts everything out
   const uint32_t t = (uint32_t)max((int)sh - 32, 0);
   uint32_t l = __funnelshift_rc(ml, mh, sh), h;
   asm("shr.u32 %0, %1, %2;" : "=r"(l) : "r"(l), "r"(t));   // (PTX shifts clamp at 32)
   asm("shr.u32 %0, %1, %2;" : "=r"(h) : "r"(mh), "r"(sh));
   const uint32_t sg = (uint32_t)((int)bh >> 31);
-  asm("add.cc.u32 %0, %2, %4;\n addc.u32 %1, %3, 0x808080;\n"
+  asm("add.cc.u32 %0, %2, %4;\n addc.u32 %1, %3, 0x40201008;\n"
       : "=r"(lo), "=r"(hi)
-      : "r"(l ^ sg), "r"(h ^ sg), "r"(0x80808080u - sg));
+      : "r"(l ^ sg), "r"(h ^ sg), "r"(0x04020100u - sg));
 }
 
-// digit bytes B of the words of two consecutive k -> two float16 digits: 1024 + byte by bit pattern, less 1152
-template <int B, bool TOP>
+// the high word of a slab value raised by 2^(sa >> 20) (sa >= 0); what leaves the range becomes an infinity, so that
+// the column takes the float64 loop; zeros and denormals stay
+__device__ __forceinline__ uint32_t raise(uint32_t bh, uint32_t sa) {
+  const uint32_t h = bh & 0x7FFFFFFFu;
+  const uint32_t t = h < 0x100000u ? h : min(h + sa, 0x7FF00000u);
+  return t | (bh & 0x80000000u);
+}
+
+// The digit in bits S .. of the 16-bit half words PRM selects from the words of two consecutive k -> two float16
+// digits: 1024 + field by bit pattern, less 1280.
+template <uint32_t PRM, int S, uint32_t MASK = 0x01FF01FFu>
 __device__ __forceinline__ uint32_t digit_pair(uint32_t a, uint32_t b) {
-  uint32_t w = TOP ? __byte_perm(a, b, 0x7632) : __byte_perm(a, b, 0x0400 + 0x1111 * B) & 0x00FF00FFu;
-  w |= 0x64006400u;
-  asm("sub.f16x2 %0, %1, %2;" : "=r"(w) : "r"(w), "r"(0x64806480u));
+  uint32_t w = ((__byte_perm(a, b, PRM) >> S) & MASK) | 0x64006400u;
+  asm("sub.f16x2 %0, %1, %2;" : "=r"(w) : "r"(w), "r"(0x65006500u));
   return w;
 }
-template <int B, bool TOP = false>
+template <uint32_t PRM, int S, uint32_t MASK = 0x01FF01FFu>
 __device__ __forceinline__ void store_digit(uint32_t addr, const uint32_t (&g)[8]) {
-  st_shared_v4(addr, digit_pair<B, TOP>(g[0], g[1]), digit_pair<B, TOP>(g[2], g[3]), digit_pair<B, TOP>(g[4], g[5]),
-               digit_pair<B, TOP>(g[6], g[7]));
+  st_shared_v4(addr, digit_pair<PRM, S, MASK>(g[0], g[1]), digit_pair<PRM, S, MASK>(g[2], g[3]),
+               digit_pair<PRM, S, MASK>(g[4], g[5]), digit_pair<PRM, S, MASK>(g[6], g[7]));
 }
 
-// sum_g 2^(8 (6 - g)) D_g 2^(ea + ec - 2154) rounded to a double, expo = (ea + ec - 1013) << 20: a fixed-point sum
-// (w2:w1 in units of D_5, four fraction bits on top of w0) in 32-bit words, no FP64
-__device__ __forceinline__ double combine(const uint32_t (&d)[kAcc], int expo) {
-  int v[5];  // exact
-#pragma unroll
-  for (int g = 0; g < 5; ++g) v[g] = __float2int_rn(__uint_as_float(d[g]));
-  // D_5 .. D_7 as one float: its rounding is 2^-24 of D_5, below 2^-54 of the row's and column's maxima (float to
-  // integer conversions run on the narrow XU pipe: six of them instead of eight)
-  const float low = fmaf(fmaf(__uint_as_float(d[7]), 0.00390625f, __uint_as_float(d[6])), 0.00390625f, __uint_as_float(d[5]));
-  const int v5 = __float2int_rn(low * 16.f);
-  int64_t t = (int64_t)v[4] * 256 + (v5 >> 4);
-  t += (int64_t)v[3] * 65536;
-  t += (int64_t)v[2] * 16777216;
-  uint32_t w0 = (uint32_t)v5 << 28, w1 = (uint32_t)t, w2 = (uint32_t)(t >> 32) + (uint32_t)(v[0] * 256 + v[1]);
+// sum_g 2^(9 (12 - g)) D_g 2^(ea + ec - 2046 - 2 bits) rounded to a double, expo = (ea + ec - 879 - 2 bits) << 20: a
+// 96-bit fixed-point sum (w2:w1:w0, in sixteenths of D_6) in integers, no FP64.  v: D_0 .. D_4, 16 (D_5 + ...)
+__device__ __forceinline__ double combine(const int (&v)[6], int expo) {
+  const int64_t mid = (int64_t)v[3] * (1ll << 31) + (int64_t)v[4] * (1 << 22) + (int64_t)v[5] * (1 << 9);
+  const int64_t top = (int64_t)v[0] * (1 << 26) + (int64_t)v[1] * (1 << 17) + (int64_t)v[2] * 256 + (mid >> 32);
+  uint32_t w0 = (uint32_t)mid, w1 = (uint32_t)top, w2 = (uint32_t)(top >> 32);
   const uint32_t s = (uint32_t)((int)w2 >> 31);
   asm("add.cc.u32 %0, %3, %6;\n addc.cc.u32 %1, %4, 0;\n addc.u32 %2, %5, 0;\n"
       : "=r"(w0), "=r"(w1), "=r"(w2)
@@ -177,6 +188,15 @@ __device__ __forceinline__ double combine(const uint32_t (&d)[kAcc], int expo) {
       : "=r"(rl), "=r"(rh)
       : "r"(__funnelshift_r(nl, nh, 11)), "r"(nh >> 11), "r"((nl >> 10) & 1u), "r"((uint32_t)(expo - lz * (1 << 20))));
   return __hiloint2double((int)(rh | (s & 0x80000000u)), (int)rl);
+}
+
+// D_0 .. D_4 as integers, D_5 + D_6 / 512 + D_7 / 512^2 in sixteenths (float32: its rounding is 2^-57 of the row's and
+// column's maxima; float to integer conversions run on the narrow XU pipe: six of them instead of eight)
+__device__ __forceinline__ void sums_of(const uint32_t (&d)[kAcc][4], int e, int (&v)[6]) {
+#pragma unroll
+  for (int g = 0; g < 5; ++g) v[g] = __float2int_rn(__uint_as_float(d[g][e]));
+  v[5] = __float2int_rn(fmaf(fmaf(__uint_as_float(d[7][e]), 0.001953125f, __uint_as_float(d[6][e])), 0.03125f,
+                             __uint_as_float(d[5][e]) * 16.f));
 }
 
 // kind::f16 with float16 A and B, float32 accumulation, M = 128, N = n
@@ -239,7 +259,9 @@ template <int NT, bool SMALL>
 __global__ void __launch_bounds__(kF64Threads, 1) k_tc_f64(const __grid_constant__ F64Args a) {
   constexpr int kRows = SMALL ? 128 : NT;          // slab columns of a tile
   constexpr int kN = SMALL ? 64 : NT;              // MMA N
-  constexpr int kCols = kAcc * kN;                 // tensor-memory columns: 512 or 256
+  constexpr int kHalf = 2;                         // NT = 32: K blocks from here on use the second accumulators
+  constexpr int kCols = kAcc * kN * (kN == 32 ? 2 : 1);  // tensor-memory columns: 512
+  constexpr int kBits = SMALL ? kBitsSmall : kBitsLarge;
   constexpr int kOct = SMALL ? 2 : 3;              // octets of eight doubles a worker holds per tile
   constexpr uint32_t kWItem = SMALL ? 64 * 128 : kBlockA;  // bytes of one TMA item of W
   extern __shared__ unsigned char t64_smem[];
@@ -380,7 +402,9 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_tc_f64(const __grid_constant
                 tc_fence_after();
                 const uint32_t alo = desc_lo(sW + s * kWItem);
                 const uint32_t blo = desc_lo(base) + (((uint32_t)kb * tileX) >> 4);
-                issue_item<kN, true>(i, tmem, alo, blo, digX >> 4, id, ks, kb == 0 && i < 2);
+                const bool second = kN == 32 && kb >= kHalf;
+                issue_item<kN, true>(i, tmem + (second ? kAcc * kN : 0), alo, blo, digX >> 4, id, ks,
+                                     (kb == 0 || (kN == 32 && kb == kHalf)) && i < 2);
                 mma_commit(empty0 + 8 * s);
               }
             }
@@ -416,13 +440,21 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_tc_f64(const __grid_constant
       int ci, slab, n0;
       locate(q, &ci, &slab, &n0);
       const F64Comp& cp = a.c[ci];
-      const int octs = ((cp.K + 63) / 64) * 8 * kRows;
+      const int octs = ((cp.K + 63) / 64) * 8 * kRows, l = mode_of(cp, slab);
       int* cmax = s_max + (si & 1) * kRows;  // high word of each column's largest magnitude (0: all zero)
       if (tid < kRows) s_max[((si + 1) & 1) * kRows + tid] = 0;  // the other buffer, for the next tile
 #pragma unroll
       for (int o = 0; o < kOct; ++o) {
         const int idx = o * kWorkers + tid;
         if (idx >= octs) break;
+        if (cp.bal) {  // balanced columns of W: the same exponents on the slab's modes
+          const int k0 = (idx / kRows) * 8;
+          const int* sa = cp.bal + (int64_t)l * cp.K;
+#pragma unroll
+          for (int e = 0; e < 8; ++e)
+            v[o][e] = __hiloint2double((int)raise((uint32_t)__double2hiint(v[o][e]), (uint32_t)sa[min(k0 + e, cp.K - 1)]),
+                                       __double2loint(v[o][e]));
+        }
         uint32_t mx = 0, low = 0;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
@@ -441,20 +473,23 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_tc_f64(const __grid_constant
         const uint32_t cm = (uint32_t)cmax[n], em = cm ? cm >> 20 : 4096u;
         uint32_t lo[8], hi[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) digits32(v[o][e], em, lo[e], hi[e]);
+        for (int e = 0; e < 8; ++e)
+          digits32<kBits>((uint32_t)__double2hiint(v[o][e]), (uint32_t)__double2loint(v[o][e]), em, lo[e], hi[e]);
         const uint32_t at = base + (uint32_t)(ko >> 3) * tileX + sw128(n, (ko & 7) * 16);
-        store_digit<2, true>(at, hi);
-        store_digit<1>(at + digX, hi);
-        store_digit<0>(at + 2 * digX, hi);
-        store_digit<3>(at + 3 * digX, lo);
-        store_digit<2>(at + 4 * digX, lo);
-        store_digit<1>(at + 5 * digX, lo);
-        store_digit<0>(at + 6 * digX, lo);
+        store_digit<0x7632, 6, 0x03FF03FFu>(at, hi);  // bits 54 .. 63
+        store_digit<0x6521, 5>(at + digX, hi);        // 45 .. 53
+        store_digit<0x5410, 4>(at + 2 * digX, hi);    // 36 .. 44
+        store_digit<0x7632, 2>(at + 4 * digX, lo);    // 18 .. 26
+        store_digit<0x6521, 1>(at + 5 * digX, lo);    // 9 .. 17
+        store_digit<0x5410, 0>(at + 6 * digX, lo);    // 0 .. 8
+#pragma unroll
+        for (int e = 0; e < 8; ++e) lo[e] = __funnelshift_r(lo[e], hi[e], 24);
+        store_digit<0x5410, 3>(at + 3 * digX, lo);    // 27 .. 35
       }
       fence_async_smem();
       mbar_arrive(bready);
       if (q + (int)gridDim.x < a.total) load_tile(q + gridDim.x);  // in flight during the MMAs
-      const int l = mode_of(cp, slab), mt = SMALL ? 1 : (cp.K + 127) / 128;
+      const int mt = SMALL ? 1 : (cp.K + 127) / 128;
       // this warp's tensor-memory lanes and columns
       const int qd = warp & 3, part = kN / (kWorkers / 128), c_lo = (warp >> 2) * part;
       double* o = cp.out + (int64_t)slab * cp.out_slab;
@@ -474,16 +509,31 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_tc_f64(const __grid_constant
           }
           for (int c0 = c_lo; c0 < c_lo + part && c0 < lim_c; c0 += 4) {
             uint32_t d[kAcc][4];
+            int vs[4][6];
+            const uint32_t at = tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)c0;
 #pragma unroll
-            for (int g = 0; g < kAcc; ++g) tmem_ld4(tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(g * kN + c0), d[g]);
+            for (int g = 0; g < kAcc; ++g) tmem_ld4(at + (uint32_t)(g * kN), d[g]);
             tmem_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sums_of(d, e, vs[e]);
+            if (kN == 32 && cp.K > 64 * kHalf) {  // the second half of K
+#pragma unroll
+              for (int g = 0; g < kAcc; ++g) tmem_ld4(at + (uint32_t)((kAcc + g) * kN), d[g]);
+              tmem_wait_ld();
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                int w2[6];
+                sums_of(d, e, w2);
+#pragma unroll
+                for (int g = 0; g < 6; ++g) vs[e][g] += w2[g];
+              }
+            }
             double res[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
               const int mc = SMALL ? m_lane : cmax[c0 + e];  // of the slab column
               const int ec = SMALL ? (c0 + e < cp.K ? cp.expA[(int64_t)l * cp.K + c0 + e] : 0) : mc >> 20;
-              const uint32_t dd[kAcc] = {d[0][e], d[1][e], d[2][e], d[3][e], d[4][e], d[5][e], d[6][e], d[7][e]};
-              res[e] = combine(dd, (e_lane + ec - 1013) * (1 << 20));
+              res[e] = combine(vs[e], (e_lane + ec - 879 - 2 * kBits) * (1 << 20));
               if ((mc >= 1701 << 20) || (mc < 346 << 20 && mc)) {  // (an all-zero column gave 0)
                 const int n = n0 + (SMALL ? r : c0 + e), rw = min(SMALL ? c0 + e : r, cp.K - 1);
                 const double* p = cp.in + (int64_t)slab * cp.in_slab + (int64_t)n * cp.sn;
@@ -550,33 +600,64 @@ __global__ void __launch_bounds__(kF64Threads, 1) k_tc_f64(const __grid_constant
   }
 }
 
-// Digits of the rows of W [rows][K]: D[((l 7 + i) M + m) ld + k] = digit i of W[l][m][k] (float16, zero for
-// k >= K), expA[row] the biased exponent of the row's maximum.  One warp per row.  'bad' is set when a row is not
-// finite or its maximum lies outside 2^+-200 (the split would not be exact; the component then keeps the
-// CUDA-core kernels).
-__global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ W, int64_t rows, int M, int ld,
-                                                    uint16_t* __restrict__ D, int* __restrict__ expA, int* bad) {
+// a_k (<< 20) of the columns of each mode's W [M][M]: the exponent of the column's maximum above the smallest one.
+// One block per mode, a thread per column.
+__global__ void __launch_bounds__(256) k_col_exponents(const double* __restrict__ W, int M, int* __restrict__ bal) {
+  __shared__ int low;
+  const double* w = W + (int64_t)blockIdx.x * M * M;
+  const int k = threadIdx.x;
+  if (k == 0) low = 2047;
+  __syncthreads();
+  uint32_t mx = 0;
+  if (k < M)
+    for (int m = 0; m < M; ++m) mx = max(mx, (uint32_t)__double2hiint(w[(int64_t)m * M + k]) & 0x7FFFFFFFu);
+  if (mx) atomicMin(&low, (int)(mx >> 20));
+  __syncthreads();
+  if (k < M) bal[(int64_t)blockIdx.x * M + k] = mx ? min((int)(mx >> 20) - low, 400) << 20 : 0;
+}
+
+// Digits of the rows of W [rows][K], its columns taken by 2^-a_k when 'bal' is given: D[((l 7 + i) M + m) ld + k] =
+// digit i of W[l][m][k] (float16, zero for k >= K), expA[row] the biased exponent of the row's maximum.  One warp per
+// row.  'bad' is set when a row is not finite or its maximum lies outside 2^+-200 (the split would not be exact), and
+// for the 59-bit integers when its digits do not keep every D_3 (and so D_0 .. D_2) within 2^24: |d_0| <= 32 and
+// |d_i| <= 256 on the slab's side, the first and second 128 of K > 192 apart.  (Digits of a matrix average half
+// their range: 0.9 x 2^24 at K = 192.)  The components then keep the CUDA-core kernels.
+__global__ void __launch_bounds__(256) k_split_rows(const double* __restrict__ W, int64_t rows, int M, int ld, int bits,
+                                                    const int* __restrict__ bal, uint16_t* __restrict__ D,
+                                                    int* __restrict__ expA, int* bad) {
   const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
+  const int64_t l = row / M, m = row - l * M;
   const double* w = W + row * M;
+  auto value = [&](int k) {
+    return bal ? w[k] * __hiloint2double((1023 << 20) - bal[l * M + k], 0) : w[k];
+  };
   uint32_t mx = 0;
-  for (int k = lane; k < M; k += 32) mx = max(mx, (uint32_t)((uint64_t)__double_as_longlong(w[k]) >> 32) & 0x7FFFFFFFu);
+  for (int k = lane; k < M; k += 32) mx = max(mx, (uint32_t)__double2hiint(value(k)) & 0x7FFFFFFFu);
   for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
   const int em = (int)(mx >> 20);
   if (lane == 0) {
     expA[row] = em;
     if (em < 823 || em > 1223) *bad = 1;
   }
-  const int64_t l = row / M, m = row - l * M;
+  int most[2] = {0, 0};  // this lane's part of the bound of D_3
   for (int k = lane; k < ld; k += 32) {
-    const uint64_t g = digits_of(k < M ? w[k] : 0.0, em);
+    const uint64_t g = digits_of(k < M ? value(k) : 0.0, em, bits);
+    int b3 = 0;
 #pragma unroll
     for (int i = 0; i < kDig; ++i) {
-      const int dg = (int)((i == 0 ? g >> 48 : (g >> (8 * (6 - i))) & 0xFFull)) - 128;
+      const int dg = (int)((i == 0 ? g >> 54 : (g >> (9 * (6 - i))) & 0x1FFull)) - 256;
       D[((l * kDig + i) * M + m) * ld + k] = __half_as_ushort(__int2half_rn(k < M ? dg : 0));
+      if (k < M && i < 4) b3 += abs(dg) * (i == 3 ? 32 : 256);
     }
+    most[M > 192 && k >= 128] += b3;
   }
+  for (int o = 16; o > 0; o >>= 1) {
+    most[0] += __shfl_xor_sync(0xffffffffu, most[0], o);
+    most[1] += __shfl_xor_sync(0xffffffffu, most[1], o);
+  }
+  if (lane == 0 && bits != kBitsSmall && max(most[0], most[1]) > 1 << 24) *bad = 1;
 }
 
 constexpr int kF64MaxK = 256;
@@ -590,16 +671,21 @@ int pad8(int n) { return (n + 7) / 8 * 8; }
 
 int64_t f64_digit_bytes(int64_t nl, int n) { return nl * n * (int64_t)(pad8(n) * kDig * 2 + 4); }
 
-// Splits W (nl matrices n x n) of a component into digits ('small': the form whose TMA box has 64 rows); *bad is
-// set when a row cannot be split exactly.
-static int split_matrix(fm_ctx* c, const double* W, int64_t nl, int n, bool small, F64Mat* f, int* bad) {
+// Splits W (nl matrices n x n) of a component into digits ('small': the form whose TMA box has 64 rows; 'balance': its
+// columns taken by powers of two); *bad is set when a row cannot be split exactly.
+static int split_matrix(fm_ctx* c, const double* W, int64_t nl, int n, bool small, bool balance, F64Mat* f, int* bad) {
   int rc;
   const int ld = pad8(n);
   void* D = nullptr;
   if ((rc = dev_alloc(c, &D, (size_t)nl * kDig * n * ld * 2))) return rc;
   if ((rc = dev_alloc(c, (void**)&f->exps, (size_t)nl * n * 4))) return rc;
+  if (balance) {
+    if ((rc = dev_alloc(c, (void**)&f->bal, (size_t)nl * n * 4))) return rc;
+    k_col_exponents<<<(unsigned)nl, 256, 0, c->stream>>>(W, n, f->bal);
+  }
   const int64_t rows = nl * n;
-  k_split_rows<<<(unsigned)((rows + 7) / 8), 256, 0, c->stream>>>(W, rows, n, ld, (uint16_t*)D, f->exps, bad);
+  k_split_rows<<<(unsigned)((rows + 7) / 8), 256, 0, c->stream>>>(W, rows, n, ld, small ? kBitsSmall : kBitsLarge, f->bal,
+                                                                  (uint16_t*)D, f->exps, bad);
   FM_CUDA(cudaGetLastError());
   f->W = W;
   if (!encode3t(&f->tm, D, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, ld, n, (int)(nl * kDig), 64, small ? 64 : 128)) return FM_ERR_CUDA;
@@ -626,10 +712,10 @@ int f64_setup(fm_ctx* c) {
   if (!all) return FM_OK;
   const bool zs = stage_k(c, 0) <= 64, xs = stage_k(c, 2) <= 64;
   for (auto& cp : c->comps) {
-    if ((rc = split_matrix(c, cp.Wzb, c->nM, cp.nz, zs, &cp.f64[0], bad)) ||
-        (rc = split_matrix(c, cp.Wz, c->nM, cp.nz, zs, &cp.f64[1], bad)) ||
-        (rc = split_matrix(c, cp.Wxb, cp.nl, cp.nx, xs, &cp.f64[2], bad)) ||
-        (rc = split_matrix(c, cp.Wx, cp.nl, cp.nx, xs, &cp.f64[3], bad)))
+    if ((rc = split_matrix(c, cp.Wzb, c->nM, cp.nz, zs, false, &cp.f64[0], bad)) ||
+        (rc = split_matrix(c, cp.Wz, c->nM, cp.nz, zs, true, &cp.f64[1], bad)) ||
+        (rc = split_matrix(c, cp.Wxb, cp.nl, cp.nx, xs, false, &cp.f64[2], bad)) ||
+        (rc = split_matrix(c, cp.Wx, cp.nl, cp.nx, xs, false, &cp.f64[3], bad)))
       return rc;
   }
   int h = 0;
@@ -658,6 +744,7 @@ int f64_stage(fm_ctx* c, int stage, const double* in, double* out) {
     f.tmA = m.tm;
     f.W = m.W;
     f.expA = m.exps;
+    f.bal = m.bal;
     f.in = in + cp.off;
     f.out = out + cp.off;
     if (stage < 2) {
