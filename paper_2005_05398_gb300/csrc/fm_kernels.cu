@@ -374,7 +374,8 @@ __global__ void __launch_bounds__(256) k_apply_z(const __grid_constant__ PlaneAr
 //     sign of s alone).  Its points are then taken in pairs (zeta, n_z - 1 - zeta) that share two evaluations
 //     instead of four.
 // He L = 0 96 x 96 x 24: 463 -> 342 us (0.95 of the FP64 pipe); J = 2..4 on mid-size grids 1.4 .. 2.1x (the sums over
-// M' in registers: their count is a template argument); He J = 10 and unequal boxes gain most from the skipped pairs.
+// M' in registers: their count is a template argument up to five components, six in the quintic basis, the longest
+// chains its y solves take).
 // ---------------------------------------------------------------------------
 template <typename T>
 struct CplSource {
@@ -403,20 +404,19 @@ struct CplArgs {
   int sdir, sq;         // float32: interval of a y base = (base + sdir) / sq
 };
 
-// the source's expansion of every M'' at point p; false outside its box
-template <int R, int NMC, typename T>
-__device__ __forceinline__ bool cpl_eval(const CplSource<T>& s, int p, int n_act, int nM, int sdir, int sq, T* E) {
-  // the M'' loop is rolled up for a count known only at run time: twelve bodies of r^3 taps gain
-  // nothing beside one (E[jM] is one store per body) and take the compiler minutes
-  constexpr int kUnM = NMC ? NMC : 1;
+// The source's expansion of every M'' at point p: ahead(M''), then take(M'', value); false outside its box.  UN: M''
+// unrolled (bodies of r^3 taps); UNZ: z taps unrolled.
+template <int R, int UN, int UNZ, typename T, typename A, typename F>
+__device__ __forceinline__ bool cpl_eval(const CplSource<T>& s, int p, int n_act, int nM, int sdir, int sq, A ahead, F take) {
   const int bz = s.base[p];
   if (bz < 0) return false;
   const int bx = s.base[n_act + p], by = s.base[2 * n_act + p];
   T vz[R], vx[R], vy[R];
   int ix[R];
+  auto zval = [&](int t) { return UNZ == R ? vz[t] : s.val[t * (int64_t)n_act + p]; };
 #pragma unroll
   for (int t = 0; t < R; ++t) {
-    vz[t] = s.val[(0 * R + t) * (int64_t)n_act + p];
+    if (UNZ == R) vz[t] = s.val[(0 * R + t) * (int64_t)n_act + p];
     vx[t] = s.val[(1 * R + t) * (int64_t)n_act + p];
     vy[t] = s.val[(2 * R + t) * (int64_t)n_act + p];
     ix[t] = min(max(bx + t, 0), s.nx - 1);
@@ -424,12 +424,12 @@ __device__ __forceinline__ bool cpl_eval(const CplSource<T>& s, int p, int n_act
   if constexpr (std::is_same<T, float>::value) {
     // regrouped by y interval: a source row's R taps are one aligned vector load
     const int my = min(max((by + sdir) / sq, 0), s.nint - 1);
-#pragma unroll kUnM
-    for (int jM = 0; jM < (NMC ? NMC : kMaxM); ++jM) {
-      if (!NMC && jM >= nM) break;
+#pragma unroll UN
+    for (int jM = 0; jM < nM; ++jM) {
+      ahead(jM);
       const float* tb = s.stage + (int64_t)jM * s.nz * s.nx * s.nint * R;
       float sz = 0.f;
-#pragma unroll
+#pragma unroll UNZ
       for (int tz = 0; tz < R; ++tz) {
         const int64_t rz = (int64_t)(bz + tz) * s.nx;
         float sx = 0.f;
@@ -449,20 +449,20 @@ __device__ __forceinline__ bool cpl_eval(const CplSource<T>& s, int p, int n_act
           }
           sx = fmaf(vx[tx], sy, sx);
         }
-        sz = fmaf(vz[tz], sx, sz);
+        sz = fmaf(zval(tz), sx, sz);
       }
-      E[jM] = sz;
+      take(jM, sz);
     }
   } else {
     int iy[R];
 #pragma unroll
     for (int t = 0; t < R; ++t) iy[t] = min(max(by + t, 0), s.ny - 1);
-#pragma unroll kUnM
-    for (int jM = 0; jM < (NMC ? NMC : kMaxM); ++jM) {
-      if (!NMC && jM >= nM) break;
+#pragma unroll UN
+    for (int jM = 0; jM < nM; ++jM) {
+      ahead(jM);
       const T* cb = s.src + (int64_t)jM * s.npts;
       T sz = 0;
-#pragma unroll
+#pragma unroll UNZ
       for (int tz = 0; tz < R; ++tz) {
         T sx = 0;
 #pragma unroll
@@ -473,80 +473,153 @@ __device__ __forceinline__ bool cpl_eval(const CplSource<T>& s, int p, int n_act
           for (int ty = 1; ty < R; ++ty) sy = fma(vy[ty], row[iy[ty]], sy);
           sx = fma(vx[tx], sy, sx);
         }
-        sz = fma(vz[tz], sx, sz);
+        sz = fma(zval(tz), sx, sz);
       }
-      E[jM] = sz;
+      take(jM, sz);
     }
   }
   return true;
 }
 
 // acc[iM] += sum_jM w[iM][jM](p) E[jM]
-template <int NMC, typename T>
-__device__ __forceinline__ void cpl_add(const T* w, int p, int n_act, int nM, const T* E, T* acc) {
+template <int NM, typename T>
+__device__ __forceinline__ void cpl_add(const T* w, int p, int n_act, const T* E, T* acc) {
 #pragma unroll
-  for (int iM = 0; iM < (NMC ? NMC : kMaxM); ++iM) {
-    if (!NMC && iM >= nM) break;
+  for (int iM = 0; iM < NM; ++iM)
 #pragma unroll
-    for (int jM = 0; jM < (NMC ? NMC : kMaxM); ++jM) {
-      if (!NMC && jM >= nM) break;
-      acc[iM] = fma(w[(int64_t)(iM * nM + jM) * n_act + p], E[jM], acc[iM]);
-    }
-  }
+    for (int jM = 0; jM < NM; ++jM) acc[iM] = fma(w[(int64_t)(iM * NM + jM) * n_act + p], E[jM], acc[iM]);
 }
 
-template <int R, int NMC, typename T>
+template <int R, int NM, typename T>
 __global__ void __launch_bounds__(128) k_apply_coupling(const __grid_constant__ CplArgs<T> a) {
-  constexpr int NA = NMC ? NMC : kMaxM;
   int ci = 0;
   while (ci + 1 < a.ncomp && (int)blockIdx.x >= a.c[ci + 1].first) ++ci;
   const CplComp<T>& c = a.c[ci];
   const int item = ((int)blockIdx.x - c.first) * blockDim.x + threadIdx.x;
-  const int nM = NMC ? NMC : a.nM;
-  T acc[NA], E[NA];
+  T acc[NM], E[NM];
+  auto eval = [&](const CplSource<T>& s, int p) {
+    return cpl_eval<R, NM, R, T>(s, p, c.n_act, NM, a.sdir, a.sq, [](int) {}, [&](int jM, T v) { E[jM] = v; });
+  };
 #pragma unroll
-  for (int m = 0; m < NA; ++m) acc[m] = (T)0;
+  for (int m = 0; m < NM; ++m) acc[m] = (T)0;
   if (!c.mirror) {
     if (item >= c.n_act) return;
     bool any = false;
     for (int s = 0; s < c.ns; ++s) {
-      if (!cpl_eval<R, NMC, T>(c.s[s], item, c.n_act, nM, a.sdir, a.sq, E)) continue;
-      cpl_add<NMC, T>(c.s[s].w, item, c.n_act, nM, E, acc);
+      if (!eval(c.s[s], item)) continue;
+      cpl_add<NM, T>(c.s[s].w, item, c.n_act, E, acc);
       any = true;
     }
     if (!any) return;
     T* y = c.y + c.act_pt[item];
 #pragma unroll
-    for (int iM = 0; iM < NA; ++iM)
-      if (iM < nM) y[(int64_t)iM * c.npts] += acc[iM];
+    for (int iM = 0; iM < NM; ++iM) y[(int64_t)iM * c.npts] += acc[iM];
     return;
   }
   // planes zeta and n_z - 1 - zeta
   const int zeta = item / c.nxy;
   if (2 * zeta >= c.nz) return;
   const int p = item, pm = item + (c.nz - 1 - 2 * zeta) * c.nxy;
-  T accm[NA];
+  T accm[NM];
 #pragma unroll
-  for (int m = 0; m < NA; ++m) accm[m] = (T)0;
+  for (int m = 0; m < NM; ++m) accm[m] = (T)0;
   bool any = false;
-  if (cpl_eval<R, NMC, T>(c.s[0], p, c.n_act, nM, a.sdir, a.sq, E)) {
-    cpl_add<NMC, T>(c.s[0].w, p, c.n_act, nM, E, acc);
-    cpl_add<NMC, T>(c.s[1].w, pm, c.n_act, nM, E, accm);
+  if (eval(c.s[0], p)) {
+    cpl_add<NM, T>(c.s[0].w, p, c.n_act, E, acc);
+    cpl_add<NM, T>(c.s[1].w, pm, c.n_act, E, accm);
     any = true;
   }
-  if (cpl_eval<R, NMC, T>(c.s[0], pm, c.n_act, nM, a.sdir, a.sq, E)) {
-    cpl_add<NMC, T>(c.s[0].w, pm, c.n_act, nM, E, accm);
-    cpl_add<NMC, T>(c.s[1].w, p, c.n_act, nM, E, acc);
+  if (eval(c.s[0], pm)) {
+    cpl_add<NM, T>(c.s[0].w, pm, c.n_act, E, accm);
+    cpl_add<NM, T>(c.s[1].w, p, c.n_act, E, acc);
     any = true;
   }
   if (!any) return;
   T *y = c.y + c.act_pt[p], *ym = c.y + c.act_pt[pm];
 #pragma unroll
-  for (int iM = 0; iM < NA; ++iM)
-    if (iM < nM) {
-      y[(int64_t)iM * c.npts] += acc[iM];
-      ym[(int64_t)iM * c.npts] += accm[iM];
+  for (int iM = 0; iM < NM; ++iM) {
+    y[(int64_t)iM * c.npts] += acc[iM];
+    ym[(int64_t)iM * c.npts] += accm[iM];
+  }
+}
+
+// The same with n_M known at run time (NA = 12; more bodies take the compiler minutes) or in double-float: one body of
+// taps, each value going straight into the sums of every M'.  Bound by latency at 128 .. 255 registers, so
+//   * the weights of an M'' are loaded before its taps (predicated, not branched over: the loads have to be in flight
+//     together);
+//   * the two points of a mirrored pair are two threads of a block: each evaluates its own position, adds it with its
+//     own weights and hands what it is worth at the other point over in shared memory.
+// Against one thread for both points with kept values and a weight loop unrolled to 12 x 12: float64 He J = 5 / 7 / 10
+// on 40 x 40 x 8 (whole application) 358 / 495 / 713 -> 322 / 434 / 610 us, He J = 10 on 58 x 58 x 6 525 -> 433 us;
+// float32 J = 8 155 -> 106 us; double-float He L = 0 96 x 96 x 24 362 -> 220 us, Ps- L = 2 242 -> 193 us, J = 6 on
+// 30 x 30 x 6 118 -> 102 us.  float64 takes the z taps in a loop (unrolled: J = 10 723 us), float32 and double-float
+// unrolled (in a loop: float32 J = 8 142 us).
+template <int R, int NA, typename T>
+__global__ void __launch_bounds__(128) k_apply_coupling_any(const __grid_constant__ CplArgs<T> a) {
+  constexpr int kUnZ = std::is_same<T, double>::value ? 1 : R;
+  __shared__ T give[NA][128];
+  __shared__ int hit[128];
+  int ci = 0;
+  while (ci + 1 < a.ncomp && (int)blockIdx.x >= a.c[ci + 1].first) ++ci;
+  const CplComp<T>& c = a.c[ci];
+  const int blk = (int)blockIdx.x - c.first, tid = threadIdx.x, nM = NA < kMaxM ? NA : a.nM;
+  int q, r = 0;  // this thread's point, the mirrored one
+  bool live;
+  if (c.mirror) {
+    const int i = blk * 64 + (tid & 63), zeta = i / c.nxy, im = i + (c.nz - 1 - 2 * zeta) * c.nxy;
+    live = 2 * zeta < c.nz;
+    q = tid < 64 ? i : im;
+    r = tid < 64 ? im : i;
+  } else {
+    q = blk * 128 + tid;
+    live = q < c.n_act;
+  }
+  T own[NA], oth[NA];
+#pragma unroll
+  for (int m = 0; m < NA; ++m) own[m] = oth[m] = (T)0;
+  bool any = false;
+  if (live) {
+    const int ns = c.mirror ? 1 : c.ns;
+    for (int s = 0; s < ns; ++s) {
+      const T *wq = c.s[s].w + q, *wr = c.s[1].w + r;
+      const int64_t row = (int64_t)nM * c.n_act;
+      T w0[NA], w1[NA];
+      any |= cpl_eval<R, 1, kUnZ, T>(
+          c.s[s], q, c.n_act, nM, a.sdir, a.sq,
+          [&](int jM) {
+#pragma unroll
+            for (int m = 0; m < NA; ++m)
+              if (m < nM) {
+                w0[m] = wq[m * row + (int64_t)jM * c.n_act];
+                if (c.mirror) w1[m] = wr[m * row + (int64_t)jM * c.n_act];
+              }
+          },
+          [&](int jM, T v) {
+#pragma unroll
+            for (int m = 0; m < NA; ++m)
+              if (m < nM) {
+                own[m] = fma(w0[m], v, own[m]);
+                if (c.mirror) oth[m] = fma(w1[m], v, oth[m]);
+              }
+          });
     }
+  }
+  if (c.mirror) {
+    hit[tid] = any;
+#pragma unroll
+    for (int m = 0; m < NA; ++m)
+      if (m < nM) give[m][tid] = oth[m];
+    __syncthreads();
+    any = any || hit[tid ^ 64];
+#pragma unroll
+    for (int m = 0; m < NA; ++m)
+      if (m < nM) own[m] = own[m] + give[m][tid ^ 64];
+  }
+  if (!live || !any) return;
+  T* y = c.y + c.act_pt[q];
+#pragma unroll
+  for (int m = 0; m < NA; ++m)
+    if (m < nM) y[(int64_t)m * c.npts] += own[m];
 }
 
 // The y coefficients of a component regrouped by y interval: T[row][m][t] = c[row][q m - d + t] for every
@@ -1970,6 +2043,7 @@ static int apply_coupling(fm_ctx* c, const T* x, T* y, bool timed) {
     prof_end(c, tk_, 0.0, bytes);
     c->launches++;
   }
+  const bool any_nM = std::is_same<T, dd>::value || c->nM > (RT == 6 ? 6 : 5);
   CplArgs<T> a;
   std::memset(&a, 0, sizeof(a));
   a.nM = c->nM;
@@ -1993,7 +2067,7 @@ static int apply_coupling(fm_ctx* c, const T* x, T* y, bool timed) {
       q.src = x + src.off; q.npts = src.npts; q.nx = src.nx; q.ny = src.ny; q.nz = src.nz; q.nint = src.ay.nint;
       if constexpr (std::is_same<T, float>::value) q.stage = c->ystage32 + src.ystage_off;
     }
-    const int64_t items = cp.cpl_mirror ? (int64_t)(cp.nz / 2) * f.nxy : cp.n_act;
+    const int64_t items = cp.cpl_mirror ? (int64_t)(cp.nz / 2) * f.nxy * (any_nM ? 2 : 1) : cp.n_act;
     grid += (int)((items + 127) / 128);
     // per evaluation 2 (R^3 + R^2 + R) flops per M'', per point and source 2 n_M^2 for the weights
     const double cfl = 2.0 * (RT * RT * RT + RT * RT + RT) * c->nM;
@@ -2003,23 +2077,40 @@ static int apply_coupling(fm_ctx* c, const T* x, T* y, bool timed) {
   }
   if (grid == 0) return FM_OK;
   const int tk_ = timed ? prof_begin(c, FM_KERNEL_COUPLING) : -1;
-  if constexpr (std::is_same<T, dd>::value) {  // any n_M: an instantiation of this type takes the compiler seconds
-    if (RT == 6) k_apply_coupling<6, 0, T><<<grid, 128, 0, c->stream>>>(a);
-    else k_apply_coupling<4, 0, T><<<grid, 128, 0, c->stream>>>(a);
+  const int key = (RT == 6 ? 16 : 0) + c->nM;
+  if constexpr (std::is_same<T, dd>::value) {
+    switch (key) {
+      case 1: k_apply_coupling_any<4, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 2: k_apply_coupling_any<4, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 3: k_apply_coupling_any<4, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 4: k_apply_coupling_any<4, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 5: k_apply_coupling_any<4, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 17: k_apply_coupling_any<6, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 18: k_apply_coupling_any<6, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 19: k_apply_coupling_any<6, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 20: k_apply_coupling_any<6, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 21: k_apply_coupling_any<6, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 22: k_apply_coupling_any<6, 6, T><<<grid, 128, 0, c->stream>>>(a); break;
+      default:
+        if (RT == 6) k_apply_coupling_any<6, kMaxM, T><<<grid, 128, 0, c->stream>>>(a);
+        else k_apply_coupling_any<4, kMaxM, T><<<grid, 128, 0, c->stream>>>(a);
+    }
   } else {
-    switch ((RT == 6 ? 8 : 0) + (c->nM <= 5 ? c->nM : 0)) {
-      case 0: k_apply_coupling<4, 0, T><<<grid, 128, 0, c->stream>>>(a); break;
+    switch (key) {
       case 1: k_apply_coupling<4, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
       case 2: k_apply_coupling<4, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
       case 3: k_apply_coupling<4, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
       case 4: k_apply_coupling<4, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
       case 5: k_apply_coupling<4, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 9: k_apply_coupling<6, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 10: k_apply_coupling<6, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 11: k_apply_coupling<6, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 12: k_apply_coupling<6, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 13: k_apply_coupling<6, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
-      default: k_apply_coupling<6, 0, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 17: k_apply_coupling<6, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 18: k_apply_coupling<6, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 19: k_apply_coupling<6, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 20: k_apply_coupling<6, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 21: k_apply_coupling<6, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
+      case 22: k_apply_coupling<6, 6, T><<<grid, 128, 0, c->stream>>>(a); break;
+      default:
+        if (RT == 6) k_apply_coupling_any<6, kMaxM, T><<<grid, 128, 0, c->stream>>>(a);
+        else k_apply_coupling_any<4, kMaxM, T><<<grid, 128, 0, c->stream>>>(a);
     }
   }
   prof_end(c, tk_, fl, by);
