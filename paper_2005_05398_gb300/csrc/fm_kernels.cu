@@ -1127,21 +1127,31 @@ __device__ void last_block_reduce(const double* partial, int nv, unsigned* count
   if (threadIdx.x == 0) *counter = 0u;
 }
 
+__device__ __forceinline__ double lane_xor(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+__device__ __forceinline__ fmi::dd lane_xor(fmi::dd v, int m) {
+  return fmi::dd(__shfl_xor_sync(0xffffffffu, v.hi, m), __shfl_xor_sync(0xffffffffu, v.lo, m));
+}
+__device__ __forceinline__ double wide(double v) { return v; }
+__device__ __forceinline__ double wide(fmi::dd v) { return (double)v.hi + (double)v.lo; }
+
 // Sums eight values over the warp's lanes, each lane keeping half of its values at every exchange: nine adds
 // instead of the 40 of eight shuffle trees.  Lane 4 u (in the bit order below) returns the sum of v[u].
-__device__ __forceinline__ double warp_sum8(double (&v)[8], int lane) {
+// S: double, or pairs of floats (48 bits) for float32 sums: twenty instructions of the FP32 pipe an add, where a
+// conversion or an add in float64 holds its pipe as long as 64 of them.
+template <typename S>
+__device__ __forceinline__ S warp_sum8(S (&v)[8], int lane) {
 #pragma unroll
   for (int h = 4; h >= 1; h >>= 1) {
     const bool up = (lane & (4 * h)) != 0;
 #pragma unroll
     for (int u = 0; u < h; ++u) {
-      const double send = up ? v[u] : v[u + h];
-      const double keep = up ? v[u + h] : v[u];
-      v[u] = keep + __shfl_xor_sync(0xffffffffu, send, 4 * h);
+      const S send = up ? v[u] : v[u + h];
+      const S keep = up ? v[u + h] : v[u];
+      v[u] = keep + lane_xor(send, 4 * h);
     }
   }
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  v[0] += lane_xor(v[0], 2);
+  v[0] += lane_xor(v[0], 1);
   return v[0];  // of vector lane >> 2
 }
 
@@ -1154,10 +1164,11 @@ __device__ __forceinline__ double warp_norm2(const double* c, int n, int lane) {
 }
 
 // The block's sums of eight vectors from its threads' values, added in warp order: thread j < nj writes out[j * ldo].
-__device__ __forceinline__ void block_sum8(double (&v)[8], int nj, double (*sh)[kRedThreads / 32], double* out, int64_t ldo) {
+template <typename S>
+__device__ __forceinline__ void block_sum8(S (&v)[8], int nj, double (*sh)[kRedThreads / 32], double* out, int64_t ldo) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const double s = warp_sum8(v, lane);
-  if ((lane & 3) == 0) sh[lane >> 2][wid] = s;
+  const S s = warp_sum8(v, lane);
+  if ((lane & 3) == 0) sh[lane >> 2][wid] = wide(s);
   __syncthreads();
   if ((int)threadIdx.x < nj) {
     double r = 0.0;
@@ -1195,8 +1206,13 @@ __device__ __forceinline__ float f64_trunc_f32(double d) {
 // LOWP: products and per-thread sums in float32 from the leading bits of the operands (relative
 // accuracy about 1e-6 of sum |V_j| |w|), for the first Gram-Schmidt pass only.
 __device__ __forceinline__ double dot2(double2 a, double2 b, double acc) { return fma(a.y, b.y, fma(a.x, b.x, acc)); }
-__device__ __forceinline__ float dot2f(double2 a, double2 b, float acc) {
-  return fmaf(f64_lead_f32(a.y), f64_lead_f32(b.y), fmaf(f64_lead_f32(a.x), f64_lead_f32(b.x), acc));
+__device__ __forceinline__ void dot2f(double2 a, double2 b, float& x, float& y) {
+  x = fmaf(f64_lead_f32(a.x), f64_lead_f32(b.x), x);
+  y = fmaf(f64_lead_f32(a.y), f64_lead_f32(b.y), y);
+}
+// four float32 sums as one pair of floats (exact to 48 bits)
+__device__ __forceinline__ fmi::dd sum4f(float a, float b, float c, float d) {
+  return (fmi::dd(a, 0.f) + fmi::dd(b, 0.f)) + (fmi::dd(c, 0.f) + fmi::dd(d, 0.f));
 }
 
 template <bool LOWP>
@@ -1222,11 +1238,11 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many(const double* __restri
       vp[u] = reinterpret_cast<const double2*>((j < nv) ? V + (int64_t)j * ldv : extra);
     }
     double acc[JT];
-    float accf[JT];
+    float accf[4][JT];
 #pragma unroll
     for (int u = 0; u < JT; ++u) {
       acc[u] = 0.0;
-      accf[u] = 0.f;
+      accf[0][u] = accf[1][u] = accf[2][u] = accf[3][u] = 0.f;
     }
     int64_t p = lo + threadIdx.x;
     for (; p + bs < hi; p += 2 * bs) {
@@ -1241,8 +1257,12 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many(const double* __restri
 #pragma unroll
       for (int u = 0; u < JT; ++u)
         if (u < nj) {
-          if (LOWP) accf[u] = dot2f(vb[u], wb, dot2f(va[u], wa, accf[u]));
-          else acc[u] = dot2(vb[u], wb, dot2(va[u], wa, acc[u]));
+          if (LOWP) {
+            dot2f(va[u], wa, accf[0][u], accf[1][u]);
+            dot2f(vb[u], wb, accf[2][u], accf[3][u]);
+          } else {
+            acc[u] = dot2(vb[u], wb, dot2(va[u], wa, acc[u]));
+          }
         }
     }
     for (; p < hi; p += bs) {
@@ -1250,7 +1270,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many(const double* __restri
 #pragma unroll
       for (int u = 0; u < JT; ++u)
         if (u < nj) {
-          if (LOWP) accf[u] = dot2f(vp[u][p], wa, accf[u]);
+          if (LOWP) dot2f(vp[u][p], wa, accf[0][u], accf[1][u]);
           else acc[u] = dot2(vp[u][p], wa, acc[u]);
         }
     }
@@ -1260,15 +1280,19 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many(const double* __restri
       for (int u = 0; u < JT; ++u)
         if (u < nj) {
           const double* vv = reinterpret_cast<const double*>(vp[u]);
-          if (LOWP) accf[u] = fmaf(f64_lead_f32(vv[e]), f64_lead_f32(w[e]), accf[u]);
+          if (LOWP) accf[3][u] = fmaf(f64_lead_f32(vv[e]), f64_lead_f32(w[e]), accf[3][u]);
           else acc[u] = fma(vv[e], w[e], acc[u]);
         }
     }
-    if (LOWP) {
+    double* out8 = partial + (int64_t)j0 * gridDim.x + blockIdx.x;
+    if constexpr (LOWP) {
+      fmi::dd both[JT];
 #pragma unroll
-      for (int u = 0; u < JT; ++u) acc[u] = (double)accf[u];
+      for (int u = 0; u < JT; ++u) both[u] = sum4f(accf[0][u], accf[1][u], accf[2][u], accf[3][u]);
+      block_sum8(both, nj, sh, out8, gridDim.x);
+    } else {
+      block_sum8(acc, nj, sh, out8, gridDim.x);
     }
-    block_sum8(acc, nj, sh, partial + (int64_t)j0 * gridDim.x + blockIdx.x, gridDim.x);
   }
   last_block_reduce(partial, nt, counter, out);
 }
@@ -1294,26 +1318,35 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many_s(const double* __rest
       vp[u] = (j < nv) ? V + (int64_t)j * ldv : extra;
     }
     double acc[JT];
-    float accf[JT];
+    float accf[4][JT];
 #pragma unroll
     for (int u = 0; u < JT; ++u) {
       acc[u] = 0.0;
-      accf[u] = 0.f;
+      accf[0][u] = accf[1][u] = accf[2][u] = accf[3][u] = 0.f;
     }
-    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-      const double wi = w[i];
+    const int64_t bs = blockDim.x;
+    for (int64_t i = lo + threadIdx.x; i < hi; i += 4 * bs) {
 #pragma unroll
-      for (int u = 0; u < JT; ++u)
-        if (u < nj) {
-          if (LOWP) accf[u] = fmaf(f64_lead_f32(vp[u][i]), f64_lead_f32(wi), accf[u]);
-          else acc[u] = fma(vp[u][i], wi, acc[u]);
-        }
-    }
-    if (LOWP) {
+      for (int t = 0; t < 4; ++t) {
+        if (i + t * bs >= hi) break;
+        const double wi = w[i + t * bs];
 #pragma unroll
-      for (int u = 0; u < JT; ++u) acc[u] = (double)accf[u];
+        for (int u = 0; u < JT; ++u)
+          if (u < nj) {
+            if (LOWP) accf[t][u] = fmaf(f64_lead_f32(vp[u][i + t * bs]), f64_lead_f32(wi), accf[t][u]);
+            else acc[u] = fma(vp[u][i + t * bs], wi, acc[u]);
+          }
+      }
     }
-    block_sum8(acc, nj, sh, partial + (int64_t)j0 * gridDim.x + blockIdx.x, gridDim.x);
+    double* out8 = partial + (int64_t)j0 * gridDim.x + blockIdx.x;
+    if constexpr (LOWP) {
+      fmi::dd both[JT];
+#pragma unroll
+      for (int u = 0; u < JT; ++u) both[u] = sum4f(accf[0][u], accf[1][u], accf[2][u], accf[3][u]);
+      block_sum8(both, nj, sh, out8, gridDim.x);
+    } else {
+      block_sum8(acc, nj, sh, out8, gridDim.x);
+    }
   }
   last_block_reduce(partial, nt, counter, out);
 }
@@ -1330,18 +1363,23 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many32(const float* __restr
   const int64_t hi = min(n, lo + chunk);
   for (int j0 = (int)blockIdx.y * JT; j0 < nv; j0 += JT * (int)gridDim.y) {
     const int nj = min(JT, nv - j0);
-    float acc[JT];
+    float acc[4][JT];
 #pragma unroll
-    for (int u = 0; u < JT; ++u) acc[u] = 0.0f;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-      const float wi = w[i];
+    for (int u = 0; u < JT; ++u) acc[0][u] = acc[1][u] = acc[2][u] = acc[3][u] = 0.0f;
+    const int64_t bs = blockDim.x;
+    for (int64_t i = lo + threadIdx.x; i < hi; i += 4 * bs) {
 #pragma unroll
-      for (int u = 0; u < JT; ++u)
-        if (u < nj) acc[u] = fmaf(V[(int64_t)(j0 + u) * ldv + i], wi, acc[u]);
+      for (int t = 0; t < 4; ++t) {
+        if (i + t * bs >= hi) break;
+        const float wi = w[i + t * bs];
+#pragma unroll
+        for (int u = 0; u < JT; ++u)
+          if (u < nj) acc[t][u] = fmaf(V[(int64_t)(j0 + u) * ldv + i + t * bs], wi, acc[t][u]);
+      }
     }
-    double accd[JT];
+    fmi::dd accd[JT];
 #pragma unroll
-    for (int u = 0; u < JT; ++u) accd[u] = (double)acc[u];
+    for (int u = 0; u < JT; ++u) accd[u] = sum4f(acc[0][u], acc[1][u], acc[2][u], acc[3][u]);
     block_sum8(accd, nj, sh, partial + (int64_t)j0 * gridDim.x + blockIdx.x, gridDim.x);
   }
   last_block_reduce(partial, nv, counter, out);
@@ -1354,7 +1392,7 @@ __global__ void __launch_bounds__(kRedThreads) k_axpy_many_norm32(const float* _
                                                                  double* __restrict__ partial, unsigned* counter,
                                                                  double* __restrict__ out) {
   __shared__ double sh[32];
-  float acc = 0.0f;
+  double acc = 0.0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
     int j = 0;
@@ -1367,9 +1405,9 @@ __global__ void __launch_bounds__(kRedThreads) k_axpy_many_norm32(const float* _
     for (; j < nv; ++j) s0 = fmaf(h[j], V[(int64_t)j * ldv + i], s0);
     const float v = fmaf(sign, (s0 + s1) + (s2 + s3), w[i]);
     w[i] = v;
-    acc = fmaf(v, v, acc);
+    acc = fma((double)v, (double)v, acc);
   }
-  const double a = block_sum((double)acc, sh);
+  const double a = block_sum(acc, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = a;
   last_block_reduce(partial, 1, counter, out);
 }
@@ -1456,16 +1494,18 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_gs_axpy(const double* __rest
       tail = 2 * npair;
       const double2* V2 = reinterpret_cast<const double2*>(V);
       for (int64_t p = i0; p < npair; p += st) {
-        float ca = 0.f, cb = 0.f;
+        float ca = 0.f, cb = 0.f, ca1 = 0.f, cb1 = 0.f;  // even and odd basis vectors
         int j = 0;
         for (; j + 7 < nv; j += 8) {
           double2 t[8];
 #pragma unroll
           for (int u = 0; u < 8; ++u) t[u] = V2[(int64_t)(j + u) * ldp + p];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) {
+          for (int u = 0; u < 8; u += 2) {
             ca = fmaf(csf[j + u], f64_trunc_f32(t[u].x), ca);
             cb = fmaf(csf[j + u], f64_trunc_f32(t[u].y), cb);
+            ca1 = fmaf(csf[j + u + 1], f64_trunc_f32(t[u + 1].x), ca1);
+            cb1 = fmaf(csf[j + u + 1], f64_trunc_f32(t[u + 1].y), cb1);
           }
         }
         for (; j < nv; ++j) {
@@ -1474,15 +1514,20 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_gs_axpy(const double* __rest
           cb = fmaf(csf[j], f64_trunc_f32(t.y), cb);
         }
         const double2 wp = reinterpret_cast<const double2*>(w)[p];
-        const double oa = (wp.x - (double)ca) * inv_nu, ob = (wp.y - (double)cb) * inv_nu;
+        const double oa = (wp.x - (double)(ca + ca1)) * inv_nu, ob = (wp.y - (double)(cb + cb1)) * inv_nu;
         reinterpret_cast<double2*>(vout)[p] = make_double2(oa, ob);
         acc = fma(ob, ob, fma(oa, oa, acc));
       }
     }
     for (int64_t i = tail + i0; i < n; i += st) {
-      float c0 = 0.f;
-      for (int j = 0; j < nv; ++j) c0 = fmaf(csf[j], f64_trunc_f32(V[(int64_t)j * ldv + i]), c0);
-      const double o = (w[i] - (double)c0) * inv_nu;
+      float c0 = 0.f, c1 = 0.f;
+      int j = 0;
+      for (; j + 1 < nv; j += 2) {
+        c0 = fmaf(csf[j], f64_trunc_f32(V[(int64_t)j * ldv + i]), c0);
+        c1 = fmaf(csf[j + 1], f64_trunc_f32(V[(int64_t)(j + 1) * ldv + i]), c1);
+      }
+      if (j < nv) c0 = fmaf(csf[j], f64_trunc_f32(V[(int64_t)j * ldv + i]), c0);
+      const double o = (w[i] - (double)(c0 + c1)) * inv_nu;
       vout[i] = o;
       acc = fma(o, o, acc);
     }
@@ -1541,8 +1586,9 @@ __global__ void __launch_bounds__(kRedThreads, 2) k_gs_axpy(const double* __rest
 // float32, coefficients, norms and reductions in float64.
 // Multi-dot: partial[j][block] of V[j] . w over 16-byte quads (n a multiple of 4, 16-byte aligned
 // vectors), eight vectors and two quads per thread and iteration, loads issued before the FMAs.
+// (a quad's products are summed by themselves: fewer roundings than one chain over the quads of a thread)
 __device__ __forceinline__ float dot4f(float4 a, float4 b, float acc) {
-  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
+  return acc + (fmaf(a.y, b.y, a.x * b.x) + fmaf(a.w, b.w, a.z * b.z));
 }
 
 __global__ void __launch_bounds__(kRedThreads) k_dot_many32v(const float* __restrict__ V, int64_t ldv, int nv,
@@ -1562,9 +1608,9 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many32v(const float* __rest
     const float4* vp[JT];
 #pragma unroll
     for (int u = 0; u < JT; ++u) vp[u] = reinterpret_cast<const float4*>(V + (int64_t)(j0 + min(u, nj - 1)) * ldv);
-    float acc[JT];
+    float acc[2][JT];
 #pragma unroll
-    for (int u = 0; u < JT; ++u) acc[u] = 0.f;
+    for (int u = 0; u < JT; ++u) acc[0][u] = acc[1][u] = 0.f;
     int64_t p = lo + threadIdx.x;
     for (; p + bs < hi; p += 2 * bs) {
       const float4 wa = w4[p], wb = w4[p + bs];
@@ -1577,17 +1623,20 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many32v(const float* __rest
         }
 #pragma unroll
       for (int u = 0; u < JT; ++u)
-        if (u < nj) acc[u] = dot4f(vb[u], wb, dot4f(va[u], wa, acc[u]));
+        if (u < nj) {
+          acc[0][u] = dot4f(va[u], wa, acc[0][u]);
+          acc[1][u] = dot4f(vb[u], wb, acc[1][u]);
+        }
     }
     for (; p < hi; p += bs) {
       const float4 wa = w4[p];
 #pragma unroll
       for (int u = 0; u < JT; ++u)
-        if (u < nj) acc[u] = dot4f(vp[u][p], wa, acc[u]);
+        if (u < nj) acc[0][u] = dot4f(vp[u][p], wa, acc[0][u]);
     }
-    double accd[JT];
+    fmi::dd accd[JT];
 #pragma unroll
-    for (int u = 0; u < JT; ++u) accd[u] = (double)acc[u];
+    for (int u = 0; u < JT; ++u) accd[u] = fmi::dd(acc[0][u], 0.f) + fmi::dd(acc[1][u], 0.f);
     block_sum8(accd, nj, sh, partial + (int64_t)j0 * gridDim.x + blockIdx.x, gridDim.x);
   }
   last_block_reduce(partial, nv, counter, out);
@@ -1857,6 +1906,8 @@ inline int grid_for(int64_t n, int threads, int cap = 152 * 16) {
 // vectors: multi-dot 228 us (252 with two blocks per SM, 294 with four), update 212 us (260 with one, 220 with
 // four).  Short vectors: 256 threads, one pass over the items, and the groups of eight vectors side by side in
 // blockIdx.y (83 k elements, 30 vectors: 16 us; 27 with the groups in turn).
+// Float32 sums: a thread has four (two over quads, each summed by itself first), so that no sum takes more roundings
+// than one of ceil(n / 155,648) items, also between the two lengths.
 struct RedShape {
   dim3 grid;
   int threads;
@@ -1869,6 +1920,17 @@ inline RedShape dot_shape(int64_t n, int nv) {
 inline RedShape upd_shape(int64_t n) {
   if (n >= 152 * 512 * 2) return {dim3(304), 512};
   return {dim3((int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 304))), 256};
+}
+// Double-float: bound by the latency of its multiply-adds (twenty dependent instructions each), so on long vectors
+// more warps: 3.7 M elements, a solve of 48 steps, multi-dots 17 ms (152 blocks of 512 threads 30 ms), updates 10.6 ms
+// (304 blocks of 512 threads 15.7 ms).
+inline RedShape dot_shape_dd(int64_t n, int nv) {
+  if (n >= 152 * 512 * 4) return {dim3(608), 256};
+  return dot_shape(n, nv);
+}
+inline RedShape upd_shape_dd(int64_t n) {
+  if (n >= 152 * 512 * 6) return {dim3((int)std::min<int64_t>((n + 255) / 256, 2432)), 256};
+  return upd_shape(n);
 }
 
 }  // namespace
@@ -2765,7 +2827,7 @@ int axpby_dd(fm_ctx* c, double a, const dd* x, double b, dd* y) {
 
 int dot_many_dd(fm_ctx* c, const dd* V, int64_t ldv, int nv, const dd* w, double* h_host) {
   if (nv < 1 || nv > kGsMaxVec) return FM_ERR_ARG;
-  const RedShape sh = dot_shape(c->N, nv);
+  const RedShape sh = dot_shape_dd(c->N, nv);
   {
     const int tk_ = prof_begin(c, FM_KERNEL_DOT);
     k_dot_many_dd<<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, w, c->N, c->red, c->gs_cnt, c->gsd);
@@ -2783,7 +2845,7 @@ int axpy_many_dd(fm_ctx* c, const dd* V, int64_t ldv, int nv, const double* h_ho
   if (nv < 1 || nv > kGsMaxVec) return FM_ERR_ARG;
   double* hd = c->red + (int64_t)c->red_blocks * 256 + 512;
   FM_CUDA(cudaMemcpyAsync(hd, h_host, nv * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-  const RedShape sh = upd_shape(c->N);
+  const RedShape sh = upd_shape_dd(c->N);
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
     k_gs_axpy_dd<2><<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, hd, w, nullptr, c->N, nullptr, nullptr, nullptr,
@@ -2803,7 +2865,7 @@ int gs_cgs2_dd(fm_ctx* c, const dd* V, int nv, dd* w, dd* vout, double* h, doubl
   double* h1 = c->gsd;
   double* h2 = c->gsd + kGsMaxVec;
   double* sc = c->gsd + 3 * kGsMaxVec;
-  const RedShape sd = dot_shape(N, nv), su = upd_shape(N);
+  const RedShape sd = dot_shape_dd(N, nv), su = upd_shape_dd(N);
   {
     const int tk_ = prof_begin(c, FM_KERNEL_DOT);
     k_dot_many_dd<<<sd.grid, sd.threads, 0, c->stream>>>(V, N, nv, w, N, c->red, c->gs_cnt, h1);
