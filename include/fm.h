@@ -21,8 +21,9 @@
  *  - All work is ordered on the context's stream (fm_opts.stream, or the legacy
  *    default stream when NULL).  fm_apply / fm_apply_S return without synchronising;
  *    fm_precond_apply synchronises when its float32 tensor-core stages ran (it reads their
- *    wait flag; the float64 form does not synchronise: a wait that expires there leaves NaN in y and is
- *    reported by the next fm_solve / fm_eigs); fm_solve / fm_eigs synchronise before they return.
+ *    wait flag); its other forms (float64, float32 on the CUDA cores) do not: a wait that expires there
+ *    leaves NaN in y and is reported by the next fm_solve / fm_eigs.  fm_solve / fm_eigs synchronise
+ *    before they return.  FM_ERR_TIMEOUT is reported once; calls after it stand for themselves.
  *  - A context is used by one host thread at a time.
  *  - Energies are in the units of the reduced-coordinate equations (Hartree for
  *    electron-mass units); box sizes R_x, R_y are in reduced Jacobi coordinates.

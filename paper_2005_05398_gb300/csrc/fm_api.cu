@@ -755,8 +755,16 @@ int fm_precond_apply(fm_ctx* c, const double* x, double* y) {
   if (!c->have_shift) return FM_ERR_NO_SHIFT;
   FM_CUDA(cudaSetDevice(c->device));
   int rc = launch_precond(c, x, y);
-  // the float64 stages are not waited for: a wait that expires there leaves NaN, reported by the next solve
+  // the other forms are not waited for: a wait that expires there leaves NaN, reported by the next solve
   return rc || !c->tc_active ? rc : tc_check(c);
+}
+
+// The result of a solve, FM_ERR_TIMEOUT when a wait expired during it or in a call before it that does not
+// synchronise (its NaN may have shown as a breakdown).
+static int report_wait(fm_ctx* c, int rc) {
+  if (rc != FM_OK && rc != FM_ERR_NOT_CONVERGED && rc != FM_ERR_BREAKDOWN && rc != FM_ERR_TIMEOUT) return rc;
+  const int tc = tc_check(c);
+  return tc ? tc : rc;
 }
 
 int fm_solve(fm_ctx* c, double E, const double* rhs, double* x, fm_info* info) {
@@ -770,10 +778,7 @@ int fm_solve(fm_ctx* c, double E, const double* rhs, double* x, fm_info* info) {
   double res = 0.0;
   rc = solve_any(c, E, rhs, x, c->opts.tol, c->opts.max_iters, &it, &rs, &res);
   FM_CUDA(cudaStreamSynchronize(c->stream));
-  if (rc == FM_OK || rc == FM_ERR_NOT_CONVERGED) {
-    const int tc = tc_check(c);
-    if (tc) rc = tc;
-  }
+  rc = report_wait(c, rc);
   if (info) {
     std::memset(info, 0, sizeof(*info));
     info->iters = it;
@@ -791,10 +796,7 @@ int fm_eigs(fm_ctx* c, double shift, int k, const double* v0, double* evals, dou
   int rc = eigs_impl(c, shift, k, v0, evals, evecs, info);
   if (c) {
     c->n_tune = 0;
-    if (rc == FM_OK || rc == FM_ERR_NOT_CONVERGED) {
-      const int tc = tc_check(c);
-      if (tc) rc = tc;
-    }
+    rc = report_wait(c, rc);
   }
   return rc;
 }

@@ -223,7 +223,7 @@ struct fm_ctx {
   bool tc_active = false;        // float32 preconditioner x / y stages on the tensor cores
   bool bf16 = false;             // ... with BF16 operands (z stages and the fused chain), else TF32
   bool f64_tc = false;           // float64 preconditioner z / x stages on the tensor cores (digit splitting)
-  int* tc_err = nullptr;         // device flag: a bounded wait of a tensor-core kernel expired
+  int* tc_err = nullptr;         // device flag: a bounded wait of a kernel expired
   int64_t launches = 0;
   int64_t device_bytes = 0;
   // per-kernel timing (fm_profile)
@@ -290,7 +290,7 @@ int prof_harvest(fm_ctx* c);   // after a stream synchronisation: fold finished 
 bool tc_component_ok(const Comp& cp);
 int tc_setup(fm_ctx* c);       // after the stage buffers exist: encode the TMA maps
 int tc_kernels_init();
-int tc_check(fm_ctx* c);       // FM_ERR_TIMEOUT when a tensor-core kernel gave up a wait
+int tc_check(fm_ctx* c);       // FM_ERR_TIMEOUT when a kernel gave up a wait since the last report; clears the flag
 int* tc_flag_slot(fm_ctx* c);  // the wait flag's place in the Gram-Schmidt result buffer (read every step)
 // tensor-core chain over all components: z and x forward (+ y for the diagonalised n_M = 1 form, fused
 // per slab where eligible); the components left for the banded y solves are returned in 'banded'

@@ -1396,7 +1396,9 @@ int tc_check(fm_ctx* c) {
   int h = 0;
   FM_CUDA(cudaMemcpyAsync(&h, c->tc_err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
   FM_CUDA(cudaStreamSynchronize(c->stream));
-  return h ? FM_ERR_TIMEOUT : FM_OK;
+  if (!h) return FM_OK;
+  FM_CUDA(cudaMemsetAsync(c->tc_err, 0, sizeof(int), c->stream));  // reported once: later calls stand for themselves
+  return FM_ERR_TIMEOUT;
 }
 
 }  // namespace fmi
