@@ -672,12 +672,18 @@ int pad8(int n) { return (n + 7) / 8 * 8; }
 int64_t f64_digit_bytes(int64_t nl, int n) { return nl * n * (int64_t)(pad8(n) * kDig * 2 + 4); }
 
 // Splits W (nl matrices n x n) of a component into digits ('small': the form whose TMA box has 64 rows; 'balance': its
-// columns taken by powers of two); *bad is set when a row cannot be split exactly.
-static int split_matrix(fm_ctx* c, const double* W, int64_t nl, int n, bool small, bool balance, F64Mat* f, int* bad) {
+// columns taken by powers of two); *bad is set when a row cannot be split exactly, *mapped cleared when the digits have
+// no tensor map.
+static int split_matrix(fm_ctx* c, const double* W, int64_t nl, int n, bool small, bool balance, F64Mat* f, int* bad,
+                        bool* mapped) {
   int rc;
   const int ld = pad8(n);
   void* D = nullptr;
   if ((rc = dev_alloc(c, &D, (size_t)nl * kDig * n * ld * 2))) return rc;
+  if (!encode3t(&f->tm, D, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, ld, n, (int)(nl * kDig), 64, small ? 64 : 128)) {
+    *mapped = false;
+    return FM_OK;
+  }
   if ((rc = dev_alloc(c, (void**)&f->exps, (size_t)nl * n * 4))) return rc;
   if (balance) {
     if ((rc = dev_alloc(c, (void**)&f->bal, (size_t)nl * n * 4))) return rc;
@@ -688,7 +694,6 @@ static int split_matrix(fm_ctx* c, const double* W, int64_t nl, int n, bool smal
                                                                   (uint16_t*)D, f->exps, bad);
   FM_CUDA(cudaGetLastError());
   f->W = W;
-  if (!encode3t(&f->tm, D, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, ld, n, (int)(nl * kDig), 64, small ? 64 : 128)) return FM_ERR_CUDA;
   return FM_OK;
 }
 
@@ -699,7 +704,8 @@ static int stage_k(const fm_ctx* c, int stage) {
   return k;
 }
 
-// FM_PREC_FP64: digits of the z and x matrices of every component they serve.
+// FM_PREC_FP64: digits of the z and x matrices of every component they serve.  Without tensor maps for them (a driver
+// without the encoder, an encoding refused) the CUDA-core kernels stay.
 int f64_setup(fm_ctx* c) {
   if (c->opts.precision != FM_PREC_FP64 || c->opts.mma == FM_MMA_SIMT) return FM_OK;
   int rc;
@@ -712,11 +718,14 @@ int f64_setup(fm_ctx* c) {
   if (!all) return FM_OK;
   const bool zs = stage_k(c, 0) <= 64, xs = stage_k(c, 2) <= 64;
   for (auto& cp : c->comps) {
-    if ((rc = split_matrix(c, cp.Wzb, c->nM, cp.nz, zs, false, &cp.f64[0], bad)) ||
-        (rc = split_matrix(c, cp.Wz, c->nM, cp.nz, zs, true, &cp.f64[1], bad)) ||
-        (rc = split_matrix(c, cp.Wxb, cp.nl, cp.nx, xs, false, &cp.f64[2], bad)) ||
-        (rc = split_matrix(c, cp.Wx, cp.nl, cp.nx, xs, false, &cp.f64[3], bad)))
-      return rc;
+    const double* W[4] = {cp.Wzb, cp.Wz, cp.Wxb, cp.Wx};
+    for (int st = 0; st < 4; ++st) {
+      bool mapped = true;
+      if ((rc = split_matrix(c, W[st], st < 2 ? c->nM : cp.nl, st < 2 ? cp.nz : cp.nx, st < 2 ? zs : xs, st == 1,
+                             &cp.f64[st], bad, &mapped)))
+        return rc;
+      if (!mapped) return FM_OK;
+    }
   }
   int h = 0;
   FM_CUDA(cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
