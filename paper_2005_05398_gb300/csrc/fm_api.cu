@@ -636,8 +636,10 @@ int fm_create(const fm_system* sys, const fm_grid* grids, int n_grids, const fm_
   } else if (o.precision == FM_PREC_MIXED) {  // float32 Krylov workspace of the mixed-precision solves
     if ((rc = dev_alloc(c, (void**)&c->V32, (size_t)(m + 1) * N * 4)) || (rc = dev_alloc(c, (void**)&c->Z32, (size_t)m * N * 4)) ||
         (rc = dev_alloc(c, (void**)&c->w32, N * 4)) || (rc = dev_alloc(c, (void**)&c->r32, N * 4)) ||
-        (rc = dev_alloc(c, (void**)&c->d32, N * 4)) || (rc = dev_alloc(c, (void**)&c->e32, N * 4)) ||
-        (rc = dev_alloc(c, (void**)&c->P32, N * 4)) || (rc = dev_alloc(c, (void**)&c->Q32, N * 4)))
+        (rc = dev_alloc(c, (void**)&c->d32, N * 4)) || (rc = dev_alloc(c, (void**)&c->e32, N * 4)))
+      return fail(rc);
+    if (!local_one_pass(c->nM, c->comps[0].r) &&
+        ((rc = dev_alloc(c, (void**)&c->P32, N * 4)) || (rc = dev_alloc(c, (void**)&c->Q32, N * 4))))
       return fail(rc);
     int64_t st = 0;  // coupling sources regrouped by y interval for the float32 gather
     for (auto& cp : c->comps) {

@@ -45,6 +45,9 @@ inline int band_kq(const Axis& ay) {
 inline int band_kl(const Axis& ay, int nc) { return nc == 1 ? band_kq(ay) : band_kq(ay) * nc + 1; }
 constexpr int kMaxBandKL = 25;  // widest banded y system the y-solve kernel takes
 
+// Whether the float32 local part runs in one pass, without scratch planes: its register planes are 2 r n_M values
+inline bool local_one_pass(int nM, int r) { return nM <= (r == 6 ? 3 : 5); }
+
 // Device-side 1D tap tables of one axis.
 struct AxisDev {
   int* base = nullptr;
@@ -175,7 +178,7 @@ struct fm_ctx {
   // workspace
   double* P = nullptr;           // [N] planes of the two-pass apply (S_x S_y c)
   double* Q = nullptr;           // [N] ((D2_x S_y + S_x D2_y) c)
-  float* P32 = nullptr; float* Q32 = nullptr;  // float32 apply scratch
+  float* P32 = nullptr; float* Q32 = nullptr;  // float32 apply scratch (two-pass form only)
   double* t64 = nullptr;         // [N] preconditioner stage buffer
   double* u64 = nullptr;
   float* t32 = nullptr;

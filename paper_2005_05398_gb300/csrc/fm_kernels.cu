@@ -1960,9 +1960,6 @@ ApplyTabs<dd> tabs_of<dd>(const Comp& cp) {
   return {cp.tdd.Sx, cp.tdd.D2x, cp.tdd.Sy, cp.tdd.D2y, cp.tdd.zt, cp.tdd.qx, cp.tdd.W, cp.tdd.iy2, cp.tdd.cval, cp.tdd.cw};
 }
 
-// largest n_M of k_apply_local per r: its register planes are 2 r n_M values
-constexpr int kLocalMaxM4 = 5, kLocalMaxM6 = 3;
-
 // The local part of the operator on every component in float32, one launch (k_apply_local).
 static int apply_local32(fm_ctx* c, double E, const float* x, float* y, bool only_S, bool timed) {
   LocalArgs a;
@@ -2187,7 +2184,7 @@ static int apply_t(fm_ctx* c, double E, const T* x, T* y, bool only_S, T* P, T* 
   int rc;
   bool one_pass = false;
   if constexpr (std::is_same<T, float>::value) {
-    one_pass = c->nM <= (c->comps[0].r == 6 ? kLocalMaxM6 : kLocalMaxM4);
+    one_pass = local_one_pass(c->nM, c->comps[0].r);
     if (one_pass && (rc = apply_local32(c, E, x, y, only_S, timed))) return rc;
   }
   if (!one_pass && (rc = apply_planes<T>(c, E, x, y, only_S, P, Q, timed))) return rc;

@@ -424,19 +424,24 @@ static bool tc_requested(const fm_ctx* c) {
   return c->opts.precision != FM_PREC_FP64 && c->opts.mma != FM_MMA_SIMT;
 }
 
+// z points symmetric about 0 to rounding, in pairs
+static bool z_mirrored(const Axis& z) {
+  if (z.n % 2 != 0) return false;
+  for (int k = 0; k < z.n; ++k)
+    if (std::fabs(z.pts[k] + z.pts[z.n - 1 - k]) > 1e-15) return false;
+  return true;
+}
+
 // Whether sources 0 and 1 of a component can share their taps: the expansion of one component at +z and, by the
 // exchange symmetry, at -z, rotations that differ in the sign of s, z points symmetric to rounding.
 static bool cp_mirror(const fm_ctx* c, const Comp& cp) {
-  if (cp.sources.size() != 2 || cp.nz % 2 != 0) return false;
+  if (cp.sources.size() != 2 || !z_mirrored(cp.az)) return false;
   const Source &a = cp.sources[0], &b = cp.sources[1];
   if (a.src != b.src || a.zsign != 1.0 || b.zsign != -1.0) return false;
   double ca, sa, cb, sb;
   rotation(c->sys.mass, a.beta, cp.label, &ca, &sa);
   rotation(c->sys.mass, b.beta, cp.label, &cb, &sb);
-  if (ca != cb || sa != -sb) return false;
-  for (int k = 0; k < cp.nz; ++k)
-    if (std::fabs(cp.az.pts[k] + cp.az.pts[cp.nz - 1 - k]) > 1e-15) return false;
-  return true;
+  return ca == cb && sa == -sb;
 }
 
 int setup_host(fm_ctx* c, const fm_grid* grids, int n_grids) {
@@ -919,8 +924,9 @@ int estimate_bytes(const fm_system* S, const fm_grid* grids, int n_grids, const 
           if (split->mode != FM_SPLIT_MERKURIEV || chi(*split, ax.pts[i], ay.pts[j]) > split->vs_cut) act += 1.0;
       act *= nz;
       const double ns = 2.0;
-      bytes += act * (4.0 + ns * (12.0 + 3.0 * R * 12.0 + nM * nM * 12.0));
-      dd_tables += act * ns * (3.0 * R + nM * nM) * 8.0;
+      const double nt = S->identical_pair == 12 && labels[ic] == 3 && z_mirrored(az) ? 1.0 : ns;  // sets of taps
+      bytes += act * (4.0 + nt * (12.0 + 3.0 * R * 12.0) + ns * nM * nM * 12.0);
+      dd_tables += act * (nt * 3.0 * R + ns * nM * nM) * 8.0;
     }
     const double nl = nM + nz - 1;
     bytes += 2.0 * nM * nz * nz * 12.0 + 2.0 * nl * nx * nx * 12.0;     // z and x decompositions
@@ -950,7 +956,8 @@ int estimate_bytes(const fm_system* S, const fm_grid* grids, int n_grids, const 
     bytes += dd_tables + n * 8.0 * ((m + 1) + m + 4);                  // double-float tables and Krylov vectors
   bytes += n * 8.0 * (5 + 2 + 2 + 16) + n * 4.0 * 2;                    // apply scratch, stage buffers, tuning
   bytes += n * 8.0 * ((m + 1) + std::max(m, ncv) + (ncv + 1));          // FGMRES and Arnoldi bases
-  if (o->precision == FM_PREC_MIXED) bytes += n * 4.0 * ((m + 1) + m + 6 + 2.5);  // + y-interval sources
+  if (o->precision == FM_PREC_MIXED)  // + scratch of the two-pass form, y-interval sources
+    bytes += n * 4.0 * ((m + 1) + m + 4 + (local_one_pass(nM, grids[0].basis ? 6 : 4) ? 0 : 2) + 2.5);
   bytes += (4.0 * 152 * 256 + 8192 + 4096) * 8.0;
   *out = (int64_t)bytes;
   return FM_OK;
