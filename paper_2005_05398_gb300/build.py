@@ -15,7 +15,9 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "libfm.so")
 BUILD = os.path.join(HERE, "_build")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-SOURCES = ["fm_api.cu", "fm_kernels.cu", "fm_tc.cu", "fm_tc64.cu", "fm_noalloc.cu", "fm_setup.cpp", "fm_dense.cpp", "fm_serve.cpp"]
+SOURCES = ["fm_coupling_64_q6.cu", "fm_coupling_64_q5.cu", "fm_coupling_64_q4.cu", "fm_coupling_64.cu", "fm_coupling_32.cu",
+           "fm_coupling_dd.cu", "fm_tc.cu", "fm_ysolve.cu", "fm_kernels.cu", "fm_api.cu", "fm_tc64.cu", "fm_noalloc.cu",
+           "fm_setup.cpp", "fm_dense.cpp", "fm_serve.cpp"]
 
 
 def nvcc():
@@ -39,7 +41,7 @@ def _compile(src, verbose):
 
 def build(verbose=False, force=False):
     srcs = [os.path.join(CSRC, s) for s in SOURCES]
-    headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
+    headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     headers.append(os.path.join(os.path.dirname(HERE), "include", "fm.h"))
     if not force and os.path.exists(OUT):
         newest = max(os.path.getmtime(p) for p in srcs + headers)

@@ -1,0 +1,5 @@
+#include "fm_coupling.cuh"
+
+namespace fmcpl {
+template void run_coupling<6, 4, double>(const CplArgs<double>&, int, cudaStream_t);
+}  // namespace fmcpl

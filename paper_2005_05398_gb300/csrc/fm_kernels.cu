@@ -17,17 +17,10 @@
 #include <type_traits>
 #include <vector>
 
+#include "fm_apply.h"
 #include "fm_internal.h"
-#include "fm_tc.h"
 
 namespace {
-
-using fmi::mbar_arrive;
-using fmi::mbar_expect_tx;
-using fmi::mbar_init;
-using fmi::mbar_wait;
-
-constexpr int kMaxM = 12;  // largest n_M (J <= 11 for tau = +1)
 
 // ---------------------------------------------------------------------------
 // The local part of the operator, y = (L - E S) c (or S c).  At a collocation point (zeta, xi, eta) of component M'
@@ -364,298 +357,6 @@ __global__ void __launch_bounds__(256) k_apply_z(const __grid_constant__ PlaneAr
 }
 
 // ---------------------------------------------------------------------------
-// V^(s) coupling (Eqs. r-form, s-rot): every active collocation point adds the other components' expansions at its
-// rotated position, r x r x r taps per source and M''.  One launch serves every component; bound by the FP64 pipe
-// (r^3 + r^2 + r multiply-adds per point, source and M''), in float32 by L1.
-//   * A (point, source) pair whose rotated position lies outside the source's box (z base -1) is passed over: the
-//     expansion is zero there.  With boxes of different sizes most pairs of the wide component are outside.
-//   * With an identical pair both sources of the third component are the same expansion, and on a z grid symmetric
-//     about 0 source 2 at (x, y, z) is source 1 at (x, y, -z) (the rotations of an exchanged pair differ in the
-//     sign of s alone).  Its points are then taken in pairs (zeta, n_z - 1 - zeta) that share two evaluations
-//     instead of four.
-// He L = 0 96 x 96 x 24: 463 -> 342 us (0.95 of the FP64 pipe); J = 2..4 on mid-size grids 1.4 .. 2.1x (the sums over
-// M' in registers: their count is a template argument up to five components, six in the quintic basis, the longest
-// chains its y solves take).
-// ---------------------------------------------------------------------------
-template <typename T>
-struct CplSource {
-  const int* base;      // [3][n_act] (z, x, y) tap bases
-  const T* val;         // [3 R][n_act]
-  const T* w;           // [nM * nM][n_act]
-  const T* src;         // the source component's coefficients
-  const T* stage;       // float32: y coefficients regrouped by y interval, [nM][nz][nx][nint_y][R]
-  int64_t npts;
-  int nx, ny, nz, nint;
-};
-template <typename T>
-struct CplComp {
-  CplSource<T> s[3];
-  T* y;
-  const int* act_pt;
-  int64_t npts;
-  int n_act, ns;
-  int mirror, nz, nxy;  // mirrored pairs of sources 0 and 1: z points, active points per z plane
-  int first;            // first block
-};
-template <typename T>
-struct CplArgs {
-  CplComp<T> c[3];
-  int ncomp, nM;
-  int sdir, sq;         // float32: interval of a y base = (base + sdir) / sq
-};
-
-// The source's expansion of every M'' at point p: ahead(M''), then take(M'', value); false outside its box.  UN: M''
-// unrolled (bodies of r^3 taps); UNZ: z taps unrolled.
-template <int R, int UN, int UNZ, typename T, typename A, typename F>
-__device__ __forceinline__ bool cpl_eval(const CplSource<T>& s, int p, int n_act, int nM, int sdir, int sq, A ahead, F take) {
-  const int bz = s.base[p];
-  if (bz < 0) return false;
-  const int bx = s.base[n_act + p], by = s.base[2 * n_act + p];
-  T vz[R], vx[R], vy[R];
-  int ix[R];
-  auto zval = [&](int t) { return UNZ == R ? vz[t] : s.val[t * (int64_t)n_act + p]; };
-#pragma unroll
-  for (int t = 0; t < R; ++t) {
-    if (UNZ == R) vz[t] = s.val[(0 * R + t) * (int64_t)n_act + p];
-    vx[t] = s.val[(1 * R + t) * (int64_t)n_act + p];
-    vy[t] = s.val[(2 * R + t) * (int64_t)n_act + p];
-    ix[t] = min(max(bx + t, 0), s.nx - 1);
-  }
-  if constexpr (std::is_same<T, float>::value) {
-    // regrouped by y interval: a source row's R taps are one aligned vector load
-    const int my = min(max((by + sdir) / sq, 0), s.nint - 1);
-#pragma unroll UN
-    for (int jM = 0; jM < nM; ++jM) {
-      ahead(jM);
-      const float* tb = s.stage + (int64_t)jM * s.nz * s.nx * s.nint * R;
-      float sz = 0.f;
-#pragma unroll UNZ
-      for (int tz = 0; tz < R; ++tz) {
-        const int64_t rz = (int64_t)(bz + tz) * s.nx;
-        float sx = 0.f;
-#pragma unroll
-        for (int tx = 0; tx < R; ++tx) {
-          const float* row = tb + ((rz + ix[tx]) * s.nint + my) * R;
-          float sy = 0.f;
-          if constexpr (R == 4) {
-            const float4 c4 = __ldg(reinterpret_cast<const float4*>(row));
-            sy = fmaf(vy[3], c4.w, fmaf(vy[2], c4.z, fmaf(vy[1], c4.y, vy[0] * c4.x)));
-          } else {
-#pragma unroll
-            for (int t = 0; t < R; t += 2) {
-              const float2 c2 = __ldg(reinterpret_cast<const float2*>(row + t));
-              sy = fmaf(vy[t + 1], c2.y, fmaf(vy[t], c2.x, sy));
-            }
-          }
-          sx = fmaf(vx[tx], sy, sx);
-        }
-        sz = fmaf(zval(tz), sx, sz);
-      }
-      take(jM, sz);
-    }
-  } else {
-    int iy[R];
-#pragma unroll
-    for (int t = 0; t < R; ++t) iy[t] = min(max(by + t, 0), s.ny - 1);
-#pragma unroll UN
-    for (int jM = 0; jM < nM; ++jM) {
-      ahead(jM);
-      const T* cb = s.src + (int64_t)jM * s.npts;
-      T sz = 0;
-#pragma unroll UNZ
-      for (int tz = 0; tz < R; ++tz) {
-        T sx = 0;
-#pragma unroll
-        for (int tx = 0; tx < R; ++tx) {
-          const T* row = cb + ((int64_t)(bz + tz) * s.nx + ix[tx]) * s.ny;
-          T sy = vy[0] * row[iy[0]];
-#pragma unroll
-          for (int ty = 1; ty < R; ++ty) sy = fma(vy[ty], row[iy[ty]], sy);
-          sx = fma(vx[tx], sy, sx);
-        }
-        sz = fma(zval(tz), sx, sz);
-      }
-      take(jM, sz);
-    }
-  }
-  return true;
-}
-
-// acc[iM] += sum_jM w[iM][jM](p) E[jM]
-template <int NM, typename T>
-__device__ __forceinline__ void cpl_add(const T* w, int p, int n_act, const T* E, T* acc) {
-#pragma unroll
-  for (int iM = 0; iM < NM; ++iM)
-#pragma unroll
-    for (int jM = 0; jM < NM; ++jM) acc[iM] = fma(w[(int64_t)(iM * NM + jM) * n_act + p], E[jM], acc[iM]);
-}
-
-template <int R, int NM, typename T>
-__global__ void __launch_bounds__(128) k_apply_coupling(const __grid_constant__ CplArgs<T> a) {
-  int ci = 0;
-  while (ci + 1 < a.ncomp && (int)blockIdx.x >= a.c[ci + 1].first) ++ci;
-  const CplComp<T>& c = a.c[ci];
-  const int item = ((int)blockIdx.x - c.first) * blockDim.x + threadIdx.x;
-  T acc[NM], E[NM];
-  auto eval = [&](const CplSource<T>& s, int p) {
-    return cpl_eval<R, NM, R, T>(s, p, c.n_act, NM, a.sdir, a.sq, [](int) {}, [&](int jM, T v) { E[jM] = v; });
-  };
-#pragma unroll
-  for (int m = 0; m < NM; ++m) acc[m] = (T)0;
-  if (!c.mirror) {
-    if (item >= c.n_act) return;
-    bool any = false;
-    for (int s = 0; s < c.ns; ++s) {
-      if (!eval(c.s[s], item)) continue;
-      cpl_add<NM, T>(c.s[s].w, item, c.n_act, E, acc);
-      any = true;
-    }
-    if (!any) return;
-    T* y = c.y + c.act_pt[item];
-#pragma unroll
-    for (int iM = 0; iM < NM; ++iM) y[(int64_t)iM * c.npts] += acc[iM];
-    return;
-  }
-  // planes zeta and n_z - 1 - zeta
-  const int zeta = item / c.nxy;
-  if (2 * zeta >= c.nz) return;
-  const int p = item, pm = item + (c.nz - 1 - 2 * zeta) * c.nxy;
-  T accm[NM];
-#pragma unroll
-  for (int m = 0; m < NM; ++m) accm[m] = (T)0;
-  bool any = false;
-  if (eval(c.s[0], p)) {
-    cpl_add<NM, T>(c.s[0].w, p, c.n_act, E, acc);
-    cpl_add<NM, T>(c.s[1].w, pm, c.n_act, E, accm);
-    any = true;
-  }
-  if (eval(c.s[0], pm)) {
-    cpl_add<NM, T>(c.s[0].w, pm, c.n_act, E, accm);
-    cpl_add<NM, T>(c.s[1].w, p, c.n_act, E, acc);
-    any = true;
-  }
-  if (!any) return;
-  T *y = c.y + c.act_pt[p], *ym = c.y + c.act_pt[pm];
-#pragma unroll
-  for (int iM = 0; iM < NM; ++iM) {
-    y[(int64_t)iM * c.npts] += acc[iM];
-    ym[(int64_t)iM * c.npts] += accm[iM];
-  }
-}
-
-// The same with n_M known at run time (NA = 12; more bodies take the compiler minutes) or in double-float: one body of
-// taps, each value going straight into the sums of every M'.  Bound by latency at 128 .. 255 registers, so
-//   * the weights of an M'' are loaded before its taps (predicated, not branched over: the loads have to be in flight
-//     together);
-//   * the two points of a mirrored pair are two threads of a block: each evaluates its own position, adds it with its
-//     own weights and hands what it is worth at the other point over in shared memory.
-// Against one thread for both points with kept values and a weight loop unrolled to 12 x 12: float64 He J = 5 / 7 / 10
-// on 40 x 40 x 8 (whole application) 358 / 495 / 713 -> 322 / 434 / 610 us, He J = 10 on 58 x 58 x 6 525 -> 433 us;
-// float32 J = 8 155 -> 106 us; double-float He L = 0 96 x 96 x 24 362 -> 220 us, Ps- L = 2 242 -> 193 us, J = 6 on
-// 30 x 30 x 6 118 -> 102 us.  float64 takes the z taps in a loop (unrolled: J = 10 723 us), float32 and double-float
-// unrolled (in a loop: float32 J = 8 142 us).
-template <int R, int NA, typename T>
-__global__ void __launch_bounds__(128) k_apply_coupling_any(const __grid_constant__ CplArgs<T> a) {
-  constexpr int kUnZ = std::is_same<T, double>::value ? 1 : R;
-  __shared__ T give[NA][128];
-  __shared__ int hit[128];
-  int ci = 0;
-  while (ci + 1 < a.ncomp && (int)blockIdx.x >= a.c[ci + 1].first) ++ci;
-  const CplComp<T>& c = a.c[ci];
-  const int blk = (int)blockIdx.x - c.first, tid = threadIdx.x, nM = NA < kMaxM ? NA : a.nM;
-  int q, r = 0;  // this thread's point, the mirrored one
-  bool live;
-  if (c.mirror) {
-    const int i = blk * 64 + (tid & 63), zeta = i / c.nxy, im = i + (c.nz - 1 - 2 * zeta) * c.nxy;
-    live = 2 * zeta < c.nz;
-    q = tid < 64 ? i : im;
-    r = tid < 64 ? im : i;
-  } else {
-    q = blk * 128 + tid;
-    live = q < c.n_act;
-  }
-  T own[NA], oth[NA];
-#pragma unroll
-  for (int m = 0; m < NA; ++m) own[m] = oth[m] = (T)0;
-  bool any = false;
-  if (live) {
-    const int ns = c.mirror ? 1 : c.ns;
-    for (int s = 0; s < ns; ++s) {
-      const T *wq = c.s[s].w + q, *wr = c.s[1].w + r;
-      const int64_t row = (int64_t)nM * c.n_act;
-      T w0[NA], w1[NA];
-      any |= cpl_eval<R, 1, kUnZ, T>(
-          c.s[s], q, c.n_act, nM, a.sdir, a.sq,
-          [&](int jM) {
-#pragma unroll
-            for (int m = 0; m < NA; ++m)
-              if (m < nM) {
-                w0[m] = wq[m * row + (int64_t)jM * c.n_act];
-                if (c.mirror) w1[m] = wr[m * row + (int64_t)jM * c.n_act];
-              }
-          },
-          [&](int jM, T v) {
-#pragma unroll
-            for (int m = 0; m < NA; ++m)
-              if (m < nM) {
-                own[m] = fma(w0[m], v, own[m]);
-                if (c.mirror) oth[m] = fma(w1[m], v, oth[m]);
-              }
-          });
-    }
-  }
-  if (c.mirror) {
-    hit[tid] = any;
-#pragma unroll
-    for (int m = 0; m < NA; ++m)
-      if (m < nM) give[m][tid] = oth[m];
-    __syncthreads();
-    any = any || hit[tid ^ 64];
-#pragma unroll
-    for (int m = 0; m < NA; ++m)
-      if (m < nM) own[m] = own[m] + give[m][tid ^ 64];
-  }
-  if (!live || !any) return;
-  T* y = c.y + c.act_pt[q];
-#pragma unroll
-  for (int m = 0; m < NA; ++m)
-    if (m < nM) y[(int64_t)m * c.npts] += own[m];
-}
-
-// The y coefficients of a component regrouped by y interval: T[row][m][t] = c[row][q m - d + t] for every
-// (M', k, i) row, interval m and tap t (0 outside the basis), so that the R taps a point of interval m
-// reads are contiguous and aligned.  One thread per (row, interval); blockIdx.y = component.
-struct StageArgs {
-  const float* c[3];
-  float* T[3];
-  int64_t rows[3];
-  int ny[3], nint[3];
-  int q, d;
-};
-template <int R>
-__global__ void __launch_bounds__(256) k_stage_ytaps(const StageArgs a) {
-  const int cq = blockIdx.y, nint = a.nint[cq], ny = a.ny[cq];
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= a.rows[cq] * nint) return;
-  const int64_t row = gid / nint;
-  const int m = (int)(gid - row * nint);
-  const float* cr = a.c[cq] + row * ny;
-  float v[R];
-#pragma unroll
-  for (int t = 0; t < R; ++t) {
-    const int j = a.q * m - a.d + t;
-    v[t] = (j >= 0 && j < ny) ? cr[j] : 0.f;
-  }
-  float* o = a.T[cq] + gid * R;
-  if constexpr (R == 4) {
-    *reinterpret_cast<float4*>(o) = make_float4(v[0], v[1], v[2], v[3]);
-  } else {
-#pragma unroll
-    for (int t = 0; t < R; t += 2) *reinterpret_cast<float2*>(o + t) = make_float2(v[t], v[t + 1]);
-  }
-}
-
-// ---------------------------------------------------------------------------
 // preconditioner: z mode product  out[l][p] = sum_k W[l][k] in[k][p] for one (component, M').
 // A CTA stages W (n_z x n_z) and an n_z x 128 column tile of the input in shared memory;
 // each thread produces the n_z outputs of its column.
@@ -777,296 +478,6 @@ __global__ void __launch_bounds__(256) k_mix(const T* __restrict__ Wall, const T
       const int rr = e % BT, cc = e / BT;
       const int gr = row0 + rr, gc = col0 + cc;
       if (gr < R && gc < C) out[so + (int64_t)gc * R + gr] = Cs[cc][rr];
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Banded y solves: one lane per (l, i_x) line of a component, 32 lines per CTA; the right-hand side of a line is the
-// M' chain of y vectors u[iM][l - M'][j][i_x] interleaved as r = j n_c + c, solved in place by the banded LU factors
-// (forward with row pivots, then backward by columns).  Bound by each line's chain of dependent rows, so a row is
-// kept short:
-//   * a producer warp feeds a ring in shared memory a few chunks of rows ahead.  The host lays the factors of a CTA's
-//     lines out contiguously per row, so a chunk is one bulk copy; the line's own values ride along by cp.async.  The
-//     solver warp only waits, multiplies and stores (it copied its own rows before: half of its instructions);
-//   * both sweeps update a window of pending rows in registers (right-looking), whose shift is the destination of the
-//     update: no moves, and one multiply-add between a row's value and the next;
-//   * the pivots of a chain of n_c components only ever swap rows of the same component: with STEP = n_c two (cubic)
-//     or four (quintic) candidates are compared instead of the whole window.  Chains whose factors pivot otherwise
-//     take STEP = 1.
-// Every wait is bounded; a wait that expires sets the context's wait flag and leaves NaN in the lines.
-// ---------------------------------------------------------------------------
-struct YArgs {
-  int nx, ny, nz, M0, nl;
-  int kq;                   // band half-width of the 1D y matrices (2 cubic, 4 quintic)
-  int64_t comp_off;
-  const int* chain_lo;   // [nl]
-  const int* chain_n;    // [nl]
-  const int* pstep;      // [nl] n_c when every pivot offset of the chain is a multiple of it, else 1
-  const int64_t* band_off;  // [nl] offset into U: [block of 32 lines][n][2 kl + 1][lines of the block, padded to 4]
-  const int64_t* lmul_off;  // [nl] offset into L: [block][n][kl + 1][lines]
-};
-
-// Row walker of a line: row r = j * n_c + c lives at P0 + c * DC + j * nx (DC the distance between the
-// chain's neighbouring M' components), stepped without divisions.
-template <typename T>
-struct RowPtr {
-  T* p;
-  int c, nc;
-  int64_t dc, nx;
-  __device__ __forceinline__ void next() {
-    p += dc;
-    if (++c == nc) {
-      c = 0;
-      p += nx - (int64_t)nc * dc;
-    }
-  }
-  __device__ __forceinline__ void prev() {
-    p -= dc;
-    if (--c < 0) {
-      c = nc - 1;
-      p -= nx - (int64_t)nc * dc;
-    }
-  }
-};
-
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(bar)
-               : "memory");
-}
-__device__ __forceinline__ int pivot_of(float v) { return __float_as_int(v); }   // an integer's bits, set by the host
-__device__ __forceinline__ int pivot_of(double v) { return __double2loint(v); }
-
-constexpr int kYStages = 3;
-
-// The ring of one CTA: kYStages stages of 'rows' factor rows (slots x wd values each) and as many line values
-template <typename T>
-struct YRing {
-  T* buf;
-  uint32_t full, empty;  // barriers [kYStages]
-  int rows, fstride;     // rows per stage; values of a stage's factor part
-  __device__ __forceinline__ T* stage(int s) const { return buf + (size_t)s * (fstride + rows * 32); }
-};
-
-// The producer's sweep: chunk ch holds rows ch * rows .. of F ([n][slots][wd], in the sweep's order) and the line
-// values of the rows that enter the solver's window 'ahead' rows after them.  Returns false when a wait expired.
-template <typename T, bool FWD>
-__device__ __forceinline__ bool y_produce(const YRing<T>& rg, const T* F, int n, int slots, int wd, int ahead,
-                                          RowPtr<T> rp, bool live, int lane, int& it) {
-  const int nch = (n + rg.rows - 1) / rg.rows;
-  int next = 0;  // rp stands on row 'next' of the sweep
-  for (int ch = 0; ch < nch; ++ch, ++it) {
-    const int st = it % kYStages, r0 = ch * rg.rows, cnt = min(rg.rows, n - r0);
-    if (it >= kYStages && !__all_sync(0xffffffffu, mbar_wait(rg.empty + 8 * st, ((uint32_t)(it / kYStages) & 1u) ^ 1u)))
-      return false;
-    T* dst = rg.stage(st);
-    const uint32_t bar = rg.full + 8 * st;
-    if (lane == 0) {
-      const uint32_t bytes = (uint32_t)(cnt * slots * wd * (int)sizeof(T));
-      mbar_expect_tx(bar, bytes);
-      bulk_load((uint32_t)__cvta_generic_to_shared(dst), F + (int64_t)r0 * slots * wd, bytes, bar);
-    }
-    while (next < r0 + ahead && next < n) {  // first chunk only: the rows the solver loads itself
-      if (FWD) rp.next();
-      else rp.prev();
-      ++next;
-    }
-    T* line = dst + rg.fstride + lane;
-    for (int q = 0; q < cnt && next < n; ++q, ++next) {
-      if (live) {
-        const uint32_t d = (uint32_t)__cvta_generic_to_shared(line + q * 32);
-        if (sizeof(T) == 8) asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(rp.p + lane) : "memory");
-        else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(rp.p + lane) : "memory");
-      }
-      if (FWD) rp.next();
-      else rp.prev();
-    }
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
-  }
-  return true;
-}
-
-// The solver's sweeps.  Forward: z_r = the pivot row's entry of the window, w <- (swapped, shifted) w - L_r z_r.
-// Backward: x_r = s_0 / pivot, s <- (shifted) s - U_r x_r with U_r[d] the coefficient of x_r in row r - d.
-template <typename T, int KL, int STEP, bool FWD>
-__device__ __forceinline__ bool y_sweep(const YRing<T>& rg, int n, int wd, int lane, int lf, bool live, RowPtr<T> rp, T* first,
-                                        int& it) {
-  constexpr int NW = FWD ? KL + 1 : 2 * KL;  // window
-  constexpr int SL = FWD ? KL + 1 : 2 * KL + 1;
-  T w[NW];
-#pragma unroll
-  for (int i = 0; i < NW; ++i) w[i] = first[i];
-  const int nch = (n + rg.rows - 1) / rg.rows;
-  for (int ch = 0; ch < nch; ++ch, ++it) {
-    const int st = it % kYStages, r0 = ch * rg.rows, cnt = min(rg.rows, n - r0);
-    if (!__all_sync(0xffffffffu, mbar_wait(rg.full + 8 * st, (uint32_t)(it / kYStages) & 1u))) return false;
-    const T* f = rg.stage(st) + lf;
-    const T* line = rg.stage(st) + rg.fstride + lane;
-#pragma unroll 2
-    for (int q = 0; q < cnt; ++q, f += SL * wd) {
-      const T in = (r0 + q + NW < n) ? line[q * 32] : (T)0;
-      if (FWD) {
-        const int p = pivot_of(f[0]);
-        const T w0 = w[0];
-        T x = w0;
-#pragma unroll
-        for (int i = STEP; i <= KL; i += STEP)
-          if (p == i) x = w[i];
-#pragma unroll
-        for (int i = 0; i < KL; ++i) {
-          T src = w[i + 1];
-          if ((i + 1) % STEP == 0 && p == i + 1) src = w0;
-          w[i] = fma(-f[(i + 1) * wd], x, src);
-        }
-        w[KL] = in;
-        if (live) rp.p[lane] = x;
-        rp.next();
-      } else {
-        const T x = w[0] * f[0];
-#pragma unroll
-        for (int i = 0; i + 1 < NW; ++i) w[i] = fma(-f[(i + 1) * wd], x, w[i + 1]);
-        w[NW - 1] = fma(-f[NW * wd], x, in);
-        if (live) rp.p[lane] = x;
-        rp.prev();
-      }
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(rg.empty + 8 * st);
-  }
-  return true;
-}
-
-// the instantiation of a chain: band half-width and pivot step (the wide bands only with step 1)
-#define FM_Y_SWITCH(GO)                              \
-  switch (kl * 16 + (step == 1 ? 1 : step)) {        \
-    case 2 * 16 + 1: GO(2, 1) break;                 \
-    case 4 * 16 + 1: GO(4, 1) break;                 \
-    case 5 * 16 + 1: GO(5, 1) break;                 \
-    case 5 * 16 + 2: GO(5, 2) break;                 \
-    case 7 * 16 + 1: GO(7, 1) break;                 \
-    case 7 * 16 + 3: GO(7, 3) break;                 \
-    case 9 * 16 + 1: GO(9, 1) break;                 \
-    case 9 * 16 + 2: GO(9, 2) break;                 \
-    case 9 * 16 + 4: GO(9, 4) break;                 \
-    case 11 * 16 + 1: GO(11, 1) break;               \
-    case 11 * 16 + 5: GO(11, 5) break;               \
-    case 13 * 16 + 1: GO(13, 1) break;               \
-    case 13 * 16 + 3: GO(13, 3) break;               \
-    case 15 * 16 + 1: GO(15, 1) break;               \
-    case 17 * 16 + 1: GO(17, 1) break;               \
-    case 17 * 16 + 4: GO(17, 4) break;               \
-    case 19 * 16 + 1: GO(19, 1) break;               \
-    case 21 * 16 + 1: GO(21, 1) break;               \
-    case 23 * 16 + 1: GO(23, 1) break;               \
-    default: GO(25, 1) break;                        \
-  }
-
-// the components of one launch (blockIdx.z selects one)
-template <typename T>
-struct YBatch {
-  YArgs a[3];
-  const T* U[3];
-  const T* L[3];
-  int* err;
-};
-
-template <typename T>
-__global__ void __launch_bounds__(64) k_ysolve(const __grid_constant__ YBatch<T> yb, int rows, int slots_max, T* __restrict__ t) {
-  extern __shared__ __align__(128) unsigned char smraw_y[];
-  __shared__ __align__(8) uint64_t bars[2 * kYStages];
-  __shared__ int failed;
-  const YArgs& a = yb.a[blockIdx.z];
-  const int il = blockIdx.y, ix0 = blockIdx.x * 32;
-  if (il >= a.nl || ix0 >= a.nx) return;  // grid sized for the largest component (uniform per CTA)
-  const int nc = a.chain_n[il], lo = a.chain_lo[il], n = nc * a.ny;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int valid = min(32, a.nx - ix0), wd = (valid + 3) & ~3;  // lines of the block, and as stored
-  const bool live = lane < valid;
-  const int lf = min(lane, wd - 1);
-  const int kl = (nc == 1) ? a.kq : a.kq * nc + 1;  // band half-width of this chain (band_kl on the host)
-  const int64_t blk = (int64_t)ix0 * n;             // full blocks before this one hold 32 lines each
-  const T* Lb = yb.L[blockIdx.z] + a.lmul_off[il] + blk * (kl + 1);
-  const T* Ub = yb.U[blockIdx.z] + a.band_off[il] + blk * (2 * kl + 1);
-  RowPtr<T> rp0;
-  rp0.p = t + a.comp_off + ((int64_t)lo * a.nz + (il - lo)) * a.ny * a.nx + ix0;  // (iM, k) = (lo, l - M0 - lo), j = 0
-  rp0.c = 0;
-  rp0.nc = nc;
-  rp0.dc = (int64_t)(a.nz - 1) * a.ny * a.nx;  // (iM + 1, k - 1) from (iM, k): row r + 1 within one j
-  rp0.nx = a.nx;
-  RowPtr<T> rpe = rp0;  // row n - 1
-  rpe.p += (int64_t)(a.ny - 1) * a.nx + (int64_t)(nc - 1) * rp0.dc;
-  rpe.c = nc - 1;
-  YRing<T> rg;
-  rg.buf = reinterpret_cast<T*>(smraw_y);
-  rg.full = (uint32_t)__cvta_generic_to_shared(bars);
-  rg.empty = rg.full + 8 * kYStages;
-  rg.rows = rows;
-  rg.fstride = rows * slots_max * 32;
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kYStages; ++s) {
-      mbar_init(rg.full + 8 * s, 33);  // the bulk copy's expect and the 32 lanes' cp.async
-      mbar_init(rg.empty + 8 * s, 1);
-    }
-    failed = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  int it = 0;
-  bool ok = true;
-  if (warp == 1) {
-    ok = y_produce<T, true>(rg, Lb, n, kl + 1, wd, kl + 1, rp0, live, lane, it);
-  } else {
-    T first[fmi::kMaxBandKL + 1];
-    const int step = a.pstep[il];
-#define FM_YF(KLV, ST)                                                                              \
-  {                                                                                                 \
-    RowPtr<T> rw = rp0;                                                                             \
-    _Pragma("unroll") for (int i = 0; i <= KLV; ++i) {                                              \
-      first[i] = (live && i < n) ? rw.p[lane] : (T)0;                                               \
-      rw.next();                                                                                    \
-    }                                                                                               \
-    ok = y_sweep<T, KLV, ST, true>(rg, n, wd, lane, lf, live, rp0, first, it);                      \
-  }
-    FM_Y_SWITCH(FM_YF)
-#undef FM_YF
-  }
-  if (!ok) failed = 1;
-  // the forward results must be in memory before the backward sweep reads them
-  __threadfence();
-  __syncthreads();
-  if (!failed) {
-    if (warp == 1) {
-      ok = y_produce<T, false>(rg, Ub, n, 2 * kl + 1, wd, 2 * kl, rpe, live, lane, it);
-    } else {
-      T first[2 * fmi::kMaxBandKL];
-      const int step = 1;
-#define FM_YB(KLV, ST)                                                                              \
-  {                                                                                                 \
-    RowPtr<T> rw = rpe;                                                                             \
-    _Pragma("unroll") for (int i = 0; i < 2 * KLV; ++i) {                                           \
-      first[i] = (live && i < n) ? rw.p[lane] : (T)0;                                               \
-      rw.prev();                                                                                    \
-    }                                                                                               \
-    ok = y_sweep<T, KLV, 1, false>(rg, n, wd, lane, lf, live, rpe, first, it);                      \
-  }
-      FM_Y_SWITCH(FM_YB)
-#undef FM_YB
-    }
-    if (!ok) failed = 1;
-  }
-  __syncthreads();
-  if (failed) {  // a wait expired: let the copies in flight land, then nothing of these lines may pass for a result
-    if (warp == 1) {
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      for (int s = 0; s < kYStages && s < it; ++s) (void)mbar_wait(rg.full + 8 * ((it - 1 - s) % kYStages), (uint32_t)((it - 1 - s) / kYStages) & 1u);
-      if (lane == 0 && yb.err) atomicExch(yb.err, 1);
-    } else if (live) {
-      RowPtr<T> rw = rp0;
-      for (int r = 0; r < n; ++r) {
-        rw.p[lane] = (T)__int_as_float(0x7FC00000);
-        rw.next();
-      }
     }
   }
 }
@@ -1937,29 +1348,6 @@ inline RedShape upd_shape_dd(int64_t n) {
 
 namespace fmi {
 
-template <typename T>
-struct ApplyTabs {
-  const T *Sx, *D2x, *Sy, *D2y, *zt, *qx, *W, *iy2, *cval, *cw;
-};
-
-template <typename T>
-static ApplyTabs<T> tabs_of(const Comp& cp);
-
-template <>
-ApplyTabs<double> tabs_of<double>(const Comp& cp) {
-  return {cp.dx.S, cp.dx.D2, cp.dy.S, cp.dy.D2, cp.zt, cp.qx, cp.W, cp.iy2, cp.cpl_val, cp.cpl_w};
-}
-
-template <>
-ApplyTabs<float> tabs_of<float>(const Comp& cp) {
-  return {cp.f32.Sx, cp.f32.D2x, cp.f32.Sy, cp.f32.D2y, cp.f32.zt, cp.f32.qx, cp.f32.W, cp.f32.iy2, cp.f32.cval, cp.f32.cw};
-}
-
-template <>
-ApplyTabs<dd> tabs_of<dd>(const Comp& cp) {
-  return {cp.tdd.Sx, cp.tdd.D2x, cp.tdd.Sy, cp.tdd.D2y, cp.tdd.zt, cp.tdd.qx, cp.tdd.W, cp.tdd.iy2, cp.tdd.cval, cp.tdd.cw};
-}
-
 // The local part of the operator on every component in float32, one launch (k_apply_local).
 static int apply_local32(fm_ctx* c, double E, const float* x, float* y, bool only_S, bool timed) {
   LocalArgs a;
@@ -2074,110 +1462,6 @@ static int apply_planes(fm_ctx* c, double E, const T* x, T* y, bool only_S, T* P
   return FM_OK;
 }
 
-// y += the V^(s) coupling of x, every component in one launch (float32: on sources regrouped by y interval first).
-template <typename T>
-static int apply_coupling(fm_ctx* c, const T* x, T* y, bool timed) {
-  const int RT = c->comps[0].r;
-  if constexpr (std::is_same<T, float>::value) {
-    StageArgs st;
-    std::memset(&st, 0, sizeof(st));
-    int64_t most = 0;
-    double bytes = 0.0;
-    for (size_t k = 0; k < c->comps.size(); ++k) {
-      const Comp& cp = c->comps[k];
-      st.c[k] = x + cp.off;
-      st.T[k] = c->ystage32 + cp.ystage_off;
-      st.rows[k] = (int64_t)c->nM * cp.nz * cp.nx;
-      st.ny[k] = cp.ny;
-      st.nint[k] = cp.ay.nint;
-      most = std::max(most, st.rows[k] * cp.ay.nint);
-      bytes += 4.0 * (double)st.rows[k] * (cp.ny + (double)cp.ay.nint * RT);
-    }
-    st.q = c->comps[0].ay.q;
-    st.d = 1;
-    const dim3 g((unsigned)((most + 255) / 256), (unsigned)c->comps.size());
-    const int tk_ = timed ? prof_begin(c, FM_KERNEL_COUPLING) : -1;
-    if (RT == 6) k_stage_ytaps<6><<<g, 256, 0, c->stream>>>(st);
-    else k_stage_ytaps<4><<<g, 256, 0, c->stream>>>(st);
-    prof_end(c, tk_, 0.0, bytes);
-    c->launches++;
-  }
-  const bool any_nM = std::is_same<T, dd>::value || c->nM > (RT == 6 ? 6 : 5);
-  CplArgs<T> a;
-  std::memset(&a, 0, sizeof(a));
-  a.nM = c->nM;
-  a.sdir = 1;
-  a.sq = c->comps[0].ay.q;
-  int grid = 0;
-  double fl = 0.0, by = 0.0;
-  for (auto& cp : c->comps) {
-    if (cp.n_act == 0 || cp.sources.empty()) continue;
-    const ApplyTabs<T> tb = tabs_of<T>(cp);
-    CplComp<T>& f = a.c[a.ncomp++];
-    f.y = y + cp.off; f.npts = cp.npts; f.n_act = cp.n_act; f.act_pt = cp.act_pt; f.ns = (int)cp.sources.size();
-    f.mirror = cp.cpl_mirror ? 1 : 0; f.nz = cp.nz; f.nxy = cp.n_act / cp.nz; f.first = grid;
-    for (int s = 0; s < f.ns; ++s) {
-      const Comp& src = c->comps[cp.sources[s].src];
-      CplSource<T>& q = f.s[s];
-      const int tab = cp.cpl_mirror ? 0 : s;  // mirrored: source 0's taps serve both
-      q.base = cp.cpl_base + (int64_t)tab * 3 * cp.n_act;
-      q.val = tb.cval + (int64_t)tab * 3 * RT * cp.n_act;
-      q.w = tb.cw + (int64_t)s * c->nM * c->nM * cp.n_act;
-      q.src = x + src.off; q.npts = src.npts; q.nx = src.nx; q.ny = src.ny; q.nz = src.nz; q.nint = src.ay.nint;
-      if constexpr (std::is_same<T, float>::value) q.stage = c->ystage32 + src.ystage_off;
-    }
-    const int64_t items = cp.cpl_mirror ? (int64_t)(cp.nz / 2) * f.nxy * (any_nM ? 2 : 1) : cp.n_act;
-    grid += (int)((items + 127) / 128);
-    // per evaluation 2 (R^3 + R^2 + R) flops per M'', per point and source 2 n_M^2 for the weights
-    const double cfl = 2.0 * (RT * RT * RT + RT * RT + RT) * c->nM;
-    fl += (double)cp.n_act * (cfl * (cp.cpl_mirror ? 1 : f.ns) + 2.0 * f.ns * c->nM * c->nM);
-    by += (double)cp.n_act * (4.0 + 2.0 * c->nM * sizeof(T) +
-                              (cp.cpl_mirror ? 1 : f.ns) * (12.0 + 3.0 * RT * sizeof(T)) + f.ns * c->nM * c->nM * sizeof(T));
-  }
-  if (grid == 0) return FM_OK;
-  const int tk_ = timed ? prof_begin(c, FM_KERNEL_COUPLING) : -1;
-  const int key = (RT == 6 ? 16 : 0) + c->nM;
-  if constexpr (std::is_same<T, dd>::value) {
-    switch (key) {
-      case 1: k_apply_coupling_any<4, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 2: k_apply_coupling_any<4, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 3: k_apply_coupling_any<4, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 4: k_apply_coupling_any<4, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 5: k_apply_coupling_any<4, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 17: k_apply_coupling_any<6, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 18: k_apply_coupling_any<6, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 19: k_apply_coupling_any<6, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 20: k_apply_coupling_any<6, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 21: k_apply_coupling_any<6, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 22: k_apply_coupling_any<6, 6, T><<<grid, 128, 0, c->stream>>>(a); break;
-      default:
-        if (RT == 6) k_apply_coupling_any<6, kMaxM, T><<<grid, 128, 0, c->stream>>>(a);
-        else k_apply_coupling_any<4, kMaxM, T><<<grid, 128, 0, c->stream>>>(a);
-    }
-  } else {
-    switch (key) {
-      case 1: k_apply_coupling<4, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 2: k_apply_coupling<4, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 3: k_apply_coupling<4, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 4: k_apply_coupling<4, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 5: k_apply_coupling<4, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 17: k_apply_coupling<6, 1, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 18: k_apply_coupling<6, 2, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 19: k_apply_coupling<6, 3, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 20: k_apply_coupling<6, 4, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 21: k_apply_coupling<6, 5, T><<<grid, 128, 0, c->stream>>>(a); break;
-      case 22: k_apply_coupling<6, 6, T><<<grid, 128, 0, c->stream>>>(a); break;
-      default:
-        if (RT == 6) k_apply_coupling_any<6, kMaxM, T><<<grid, 128, 0, c->stream>>>(a);
-        else k_apply_coupling_any<4, kMaxM, T><<<grid, 128, 0, c->stream>>>(a);
-    }
-  }
-  prof_end(c, tk_, fl, by);
-  c->launches++;
-  FM_CUDA(cudaGetLastError());
-  return FM_OK;
-}
-
 // y = (H - E S) x (only_S: y = S x) in the element type T; scratch planes P and Q for the two-pass local form.
 template <typename T>
 static int apply_t(fm_ctx* c, double E, const T* x, T* y, bool only_S, T* P, T* Q, bool timed) {
@@ -2204,51 +1488,6 @@ int launch_apply32(fm_ctx* c, double E, const float* x, float* y, bool only_S) {
 // launch_apply; no per-kernel timing.
 int launch_apply_scratch(fm_ctx* c, double E, const double* x, double* y, double* P, double* Q) {
   return apply_t<double>(c, E, x, y, false, P, Q, false);
-}
-
-// Banded y solves (Eq. prec-2 y stage with the M' chain) of the given components in one launch,
-// in place on u[slab][j][i].
-template <typename T>
-static int ysolve_banded(fm_ctx* c, const std::vector<fmi::Comp*>& comps, T* u) {
-  if (comps.empty()) return FM_OK;
-  if (comps.size() > 3) return FM_ERR_ARG;
-  const double ts = (double)sizeof(T);
-  double yfl = 0.0, yby = 0.0;  // per line 2n(kl + ku + kl) + n flops; factor and vector bytes
-  YBatch<T> yb;
-  std::memset(&yb, 0, sizeof(yb));
-  yb.err = c->tc_err;
-  int slots = 5, gx = 1, gy = 1, ctas = 0;
-  for (size_t q = 0; q < comps.size(); ++q) {
-    const fmi::Comp& cp = *comps[q];
-    for (int il = 0; il < cp.nl; ++il) {
-      const int nc = cp.chain_n[il], n = nc * cp.ny, kl = band_kl(cp.ay, nc);
-      yfl += (double)cp.nx * (2.0 * n * (3.0 * kl) + n);
-      yby += (double)cp.nx * ((double)n * (3.0 * kl + 2.0) * ts + 2.0 * n * ts);
-      slots = std::max(slots, 2 * kl + 1);
-    }
-    YArgs& ya = yb.a[q];
-    ya.nx = cp.nx; ya.ny = cp.ny; ya.nz = cp.nz; ya.M0 = c->M0; ya.nl = cp.nl; ya.comp_off = cp.off;
-    ya.kq = band_kq(cp.ay);
-    ya.chain_lo = (const int*)cp.d_chain_lo; ya.chain_n = (const int*)cp.d_chain_n;
-    ya.pstep = cp.d_pstep;
-    ya.band_off = cp.d_band_off; ya.lmul_off = cp.d_lmul_off;
-    yb.U[q] = std::is_same<T, double>::value ? (const T*)cp.yU : (const T*)cp.yU32;
-    yb.L[q] = std::is_same<T, double>::value ? (const T*)cp.yL : (const T*)cp.yL32;
-    gx = std::max(gx, (cp.nx + 31) / 32);
-    gy = std::max(gy, cp.nl);
-    ctas += ((cp.nx + 31) / 32) * cp.nl;
-  }
-  // Rows per stage: as many CTAs per SM as the grid gives it (up to 8) share 220 KB; 2 to 16 rows a stage
-  const size_t per_row = (size_t)(slots + 1) * 32 * sizeof(T);
-  const int per_sm = std::max(1, std::min(8, (ctas + 151) / 152));
-  const int rows = (int)std::max<size_t>(2, std::min<size_t>(16, (220 * 1024 / per_sm - 1024) / (kYStages * per_row)));
-  const size_t sm = kYStages * rows * per_row;
-  const int tk_ = prof_begin(c, FM_KERNEL_YSOLVE);
-  k_ysolve<T><<<dim3(gx, gy, (unsigned)comps.size()), 64, sm, c->stream>>>(yb, rows, slots, u);
-  prof_end(c, tk_, yfl, yby);
-  c->launches++;
-  FM_CUDA(cudaGetLastError());
-  return FM_OK;
 }
 
 // y = P^{-1} x (Eq. prec-2), stage-major over the components: every component's z and x forward
@@ -2917,9 +2156,8 @@ int kernels_init(fm_ctx* c) {
   FM_CUDA(cudaFuncSetAttribute(k_zmix<double, float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   FM_CUDA(cudaFuncSetAttribute(k_zmix<float, double, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   FM_CUDA(cudaFuncSetAttribute(k_zmix<float, float, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  FM_CUDA(cudaFuncSetAttribute(k_ysolve<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024));
-  FM_CUDA(cudaFuncSetAttribute(k_ysolve<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 224 * 1024));
-  return tc_kernels_init();
+  int rc = ysolve_init();
+  return rc ? rc : tc_kernels_init();
 }
 
 int fill_normal(fm_ctx* c, double* x, uint64_t seed) {
