@@ -796,7 +796,7 @@ __global__ void __launch_bounds__(kRedThreads) k_dot_many32(const float* __restr
   last_block_reduce(partial, nv, counter, out);
 }
 
-// float32: w += sign * sum_j h[j] V[j], partial[block] = sum of the new w^2 (float64)
+// float32: w += sign * sum_j h[j] V[j]; with 'out', partial[block] = sum of the new w^2 (float64)
 __global__ void __launch_bounds__(kRedThreads) k_axpy_many_norm32(const float* __restrict__ V, int64_t ldv, int nv,
                                                                  const float* __restrict__ h, float sign,
                                                                  float* __restrict__ w, int64_t n,
@@ -816,8 +816,9 @@ __global__ void __launch_bounds__(kRedThreads) k_axpy_many_norm32(const float* _
     for (; j < nv; ++j) s0 = fmaf(h[j], V[(int64_t)j * ldv + i], s0);
     const float v = fmaf(sign, (s0 + s1) + (s2 + s3), w[i]);
     w[i] = v;
-    acc = fma((double)v, (double)v, acc);
+    if (out) acc = fma((double)v, (double)v, acc);
   }
+  if (!out) return;
   const double a = block_sum(acc, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = a;
   last_block_reduce(partial, 1, counter, out);
@@ -1965,7 +1966,7 @@ int axpy_many_norm32(fm_ctx* c, const float* V, int64_t ldv, int nv, const doubl
   {
     const int tk_ = prof_begin(c, FM_KERNEL_AXPY);
     k_axpy_many_norm32<<<sh.grid, sh.threads, 0, c->stream>>>(V, ldv, nv, hd, sign, w, c->N, c->red, c->gs_cnt,
-                                                          c->gsd + 3 * kGsMaxVec);
+                                                              nrm2_out ? c->gsd + 3 * kGsMaxVec : nullptr);
     prof_end(c, tk_, (2.0 * nv + 2.0) * (double)c->N, (nv + 2.0) * 4.0 * (double)c->N);
   }
   c->launches++;
