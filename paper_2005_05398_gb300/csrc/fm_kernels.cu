@@ -3,11 +3,10 @@
 //  * operator apply y = (H - E S) x (Eq. FM-lin; H from Eq. FM-pre, storage idea of
 //    Eq. l-form): sum-factorised banded contractions in y, x and z with the pointwise
 //    coefficients and the M' +- 1 couplings, one kernel that walks the z planes;
-//  * the V^(s) coupling term (Eqs. r-form, s-rot): a gather of the source
-//    component's spline coefficients at the rotated collocation points;
-//  * the tensor-trick preconditioner (Eq. prec-2): z and x mode products and the
-//    banded y solves that replace the y eigen-transforms and the tridiagonal M'
-//    chains (the same operator, factorised by banded LU);
+//    (the V^(s) coupling term of Eqs. r-form, s-rot is in fm_coupling.cuh);
+//  * the tensor-trick preconditioner (Eq. prec-2): its chain and the CUDA-core z and x
+//    mode products (the banded y solves that replace the y eigen-transforms and the
+//    tridiagonal M' chains, the same operator factorised by banded LU, are in fm_ysolve.cu);
 //  * deterministic Krylov reductions (fixed grid, fixed reduction order).
 #include <cuda_runtime.h>
 #include <stdint.h>

@@ -20,8 +20,8 @@
 // the exponent of that column's maximum: an integer add per value.
 // Accuracy, against 64-bit-mantissa sums of the solver's own matrices, over both bases, J <= 10, n_z = 8 .. 130,
 // n_x = 48 .. 256, with random and with smooth vectors taken through the chain (relative 2-norm per M' component):
-// z stages 3e-17 .. 1e-16 where the float64 chain has 6e-17 .. 1.7e-15 (K > 64: up to 1.6e-15 against 2.3e-15), x
-// stages 5e-17 .. 1.3e-15 against 1e-16 .. 1.6e-15.  The bound is normwise: an entry far below its column's largest
+// z stages 3e-17 .. 9e-17 where the float64 chain has 5e-17 .. 1.7e-15 (K > 64: up to 2e-15 against 8e-15), x
+// stages 3e-17 .. 6e-16 against 1e-16 .. 1.6e-15.  The bound is normwise: an entry far below its column's largest
 // product carries that product's last bits.  A column with an infinity, a NaN or a maximum outside 2^+-677 takes a
 // float64 loop over the original values instead.
 //
@@ -33,9 +33,10 @@
 //     128-row operand 50 of 128 rows were used and a z stage took 90 us instead of 32.)
 //   * otherwise A = 128 rows of W streamed through a ring, B = NT columns of the slab: NT = 64 fills the tensor
 //     memory (8 x 64 columns); K > 192 takes NT = 32 so that the digits fit in shared memory.
-// Bound: the MMAs (6 KB of shared-memory operands per 128 x 64 x 16: 2/3 of the time at K = 192) and the integer
-// work of split and epilogue.  Measured per stage: K = 192, 100 slabs of 192 columns 100 us (k_mix 600 us a
-// component and stage, 1.2 ms both); K = 50, 36,864 columns 32 us (k_zmix 175 us).  Every wait is bounded; a wait
+// Bound: the MMAs' shared-memory operands (6 KB per 128 x 64 x 16, 48 cycles to read for 32 of the tensor pipe, which
+// ncu shows active for 26 % of the cycles at K = 192 and 15 % at K = 50) and the integer work of split and epilogue.
+// Measured per stage, both components of He L = 0: K = 192, 100 slabs of 192 columns 104 us forward and 112 us inverse
+// (k_mix 1.2 ms); K = 50, two of 36,864 columns 60 us (k_zmix 350 us).  Every wait is bounded; a wait
 // that expires sets the context's wait flag and leaves NaN in what the CTA had to write.
 #include <cuda.h>
 #include <cuda_fp16.h>
