@@ -16,7 +16,8 @@ pytestmark = pytest.mark.gpu
 CASES = [((6, 9, 3), 0, 0, 20.0), ((8, 7, 8), 0, 2, 20.0), ((10, 6, 24), 0, 1, 20.0), ((6, 8, 12), 0, 10, 20.0),
          ((5, 6, 31), 0, 0, 20.0), ((5, 6, 32), 0, 1, 20.0), ((4, 4, 63), 0, 0, 20.0), ((3, 4, 8), 1, 4, 12.0),
          ((6, 4, 7), 1, 2, 20.0), ((33, 16, 1), 0, 0, 40.0), ((64, 12, 1), 0, 1, 80.0), ((96, 10, 1), 0, 0, 40.0),
-         ((97, 9, 1), 0, 0, 40.0), ((128, 12, 1), 0, 0, 40.0), ((55, 6, 1), 1, 1, 45.0)]
+         ((97, 9, 1), 0, 0, 40.0), ((128, 12, 1), 0, 0, 40.0), ((55, 6, 1), 1, 1, 45.0),
+         ((9, 8, 33), 0, 1, (20.0, (10, 6, 4))), ((128, 5, 2), 0, 0, (40.0, (50, 7, 5)))]  # (component 3's own grid)
 
 
 @pytest.fixture(scope="module")
@@ -73,7 +74,10 @@ class Stage:
 
 @pytest.mark.parametrize("n,basis,J,R", CASES)
 def test_no_less_accurate_than_the_float64_chain(pkg, n, basis, J, R):
+    R, n3 = R if isinstance(R, tuple) else (R, None)
     wl = make_workload("He", J, nint=n, R=(R, 17.0), basis=basis)
+    if n3:
+        wl["grids"] = {1: {"nint": n, "R": (R, 17.0)}, 3: {"nint": n3, "R": (9.0, 8.0)}}
     ctx = pkg.Context(wl, restart_m=2, ncv=3)
     rng = np.random.default_rng(sum(n) + J)
     stages = [Stage(pkg, ctx, s) for s in range(4)]
